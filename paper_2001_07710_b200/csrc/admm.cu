@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kAssignThreads) k_assign_count(const float* __
 
 // The K_out most frequent masks stay (equal counts: the lower id), in the order they have in the library.  One block:
 // thread j ranks mask j among all masks, the survivors are written in id order.
-__global__ void __launch_bounds__(256) k_pick_survivors(MaskTable lib, const unsigned long long* __restrict__ counts,
+__global__ void __launch_bounds__(256) k_pick_survivors(MaskTable lib, const unsigned long long* counts,
                                                         int K_out, unsigned short* __restrict__ masks_out) {
   pdl_wait();
   __shared__ unsigned long long s_c[kMaxK + 1];

@@ -122,6 +122,10 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 #ifdef __CUDACC__
 // After the wait the kernel's own dependents may be launched: they wait here in turn (for the whole of this kernel), and
 // everything before it has completed.
+// A kernel that starts this way may be resident while the one before it still writes, so what it reads after the wait does
+// not go through the read-only path (no __ldg, no const __restrict__ parameter), whose data must not change while a kernel
+// runs.  Open to that path is what was complete before the kernel could start: the inputs of a call that its first kernel
+// has waited for.
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(RP_THREADS) k_reduce_parts_f32(const Params p)
   const int lane = threadIdx.x & 31, slot = threadIdx.x >> 5;
   const float* src = p.partials + (size_t)li * p.parts * PIECE_FLOATS + ((size_t)slot * (TR4 * TC) + v) * 32 + lane;
   float sum = 0.0f;
-  for (int q = 0; q < p.parts; ++q) sum += __ldg(src + (size_t)q * PIECE_FLOATS);   // piece 0 first
+  for (int q = 0; q < p.parts; ++q) sum += src[(size_t)q * PIECE_FLOATS];   // piece 0 first
   const int txe_shift = (p.TXe == 4) ? 2 : (p.TXe == 2 ? 1 : 0);
   const int ly = lane >> 2, lx = lane & 3;
   const int b = (ly < it.n0) ? 0 : 1;
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(RP_THREADS) k_reduce_parts_f32(const Params p)
   const int n_img = ig * p.NI + ni;
   const int row = TR4 * ty + v / TC, col = (it.cg * p.TXe + tx) * TC + v % TC;
   if (!((b == 0 || it.band1) && ig < p.NIG && n_img < p.N) || row >= p.H || col >= p.W) return;
-  p.y[(((size_t)n_img * p.Ho + row) * p.Wo + col) * p.F + __ldg(p.xfilt + g * FG + slot)] = p.relu ? fmaxf(sum, 0.0f) : sum;
+  p.y[(((size_t)n_img * p.Ho + row) * p.Wo + col) * p.F + p.xfilt[g * FG + slot]] = p.relu ? fmaxf(sum, 0.0f) : sum;
 }
 
 // The same for a call with rectifier and 2 x 2 max pooling: one block per (cut item, pooled value of the thread
@@ -607,7 +607,7 @@ __global__ void __launch_bounds__(RP_THREADS) k_reduce_parts_pool_f32(const Para
   for (int w = 0; w < 4; ++w) {
     const float* s = src + (size_t)((2 * yy + (w >> 1)) * TC + 2 * xx + (w & 1)) * 32;
     float sum = 0.0f;
-    for (int q = 0; q < p.parts; ++q) sum += __ldg(s + (size_t)q * PIECE_FLOATS);   // piece 0 first
+    for (int q = 0; q < p.parts; ++q) sum += s[(size_t)q * PIECE_FLOATS];   // piece 0 first
     m = fmaxf(m, sum);
   }
   const int txe_shift = (p.TXe == 4) ? 2 : (p.TXe == 2 ? 1 : 0);
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(RP_THREADS) k_reduce_parts_pool_f32(const Para
   const int n_img = ig * p.NI + ni;
   const int prow = (TR4 / 2) * ty + yy, pcol = ((it.cg * p.TXe + tx) * TC >> 1) + xx;
   if (!((b == 0 || it.band1) && ig < p.NIG && n_img < p.N) || prow >= p.Ho || pcol >= p.Wo) return;
-  p.y[(((size_t)n_img * p.Ho + prow) * p.Wo + pcol) * p.F + __ldg(p.xfilt + g * FG + slot)] = m;
+  p.y[(((size_t)n_img * p.Ho + prow) * p.Wo + pcol) * p.F + p.xfilt[g * FG + slot]] = m;
 }
 
 // ------------------------------------------------------------------------------------------ host side

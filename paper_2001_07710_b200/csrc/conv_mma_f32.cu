@@ -168,9 +168,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
             v[j][0] = make_float4(0.f, 0.f, 0.f, 0.f);
             v[j][1] = v[j][0];
             if (((valid >> (4 * j + pl)) & 1u) && c < p.C) {
+              // not through the read-only path: the kernel that writes x may still run when this block starts
               const float4* src = reinterpret_cast<const float4*>(p.x + (size_t)(base[j] + shift) * p.C + c);
-              v[j][0] = __ldg(src);
-              v[j][1] = __ldg(src + 1);
+              v[j][0] = src[0];
+              v[j][1] = src[1];
             }
           }
           if (!mbar_wait<20>(empty_a(slot), par, abort_flag, p.wait_ns)) alive = false;

@@ -56,7 +56,7 @@ __host__ __device__ inline BlobPtrs blob_ptrs(void* blob, const BlobLayout& L, i
 }
 
 // One block per original filter: per-pattern counts and kept count.
-__global__ void __launch_bounds__(256) k_pack_count(const uint8_t* __restrict__ pid, int C, int K, BlobPtrs bp, int* status) {
+__global__ void __launch_bounds__(256) k_pack_count(const uint8_t* pid, int C, int K, BlobPtrs bp, int* status) {
   pdl_wait();
   extern __shared__ int sh[];   // K counters
   const int f = blockIdx.x;

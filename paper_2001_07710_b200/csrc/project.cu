@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kZeroThreads) k_zero_counters(unsigned int* hi
 constexpr int kPatBlock = 512;
 constexpr int kSelSlots = 256;               // shared-memory counters, indexed by the digit's low bits and tagged with the digit
 static_assert(kSelSlots == kCoarse && kPatBlock >= kCoarse, "one counter of each kind per thread of the first 256");
-__global__ void __launch_bounds__(kPatBlock) k_select_pattern(const float* __restrict__ w, int64_t FC, MaskTable lib,
+__global__ void __launch_bounds__(kPatBlock) k_select_pattern(const float* w, int64_t FC, MaskTable lib,
                                                               unsigned long long* __restrict__ key, unsigned char* __restrict__ pid,
                                                               unsigned int* hist, bool do_select) {
   if (!do_select) pdl_wait();                // no kernel of this call before this one
@@ -197,10 +197,10 @@ __global__ void __launch_bounds__(kPatBlock) k_select_pattern(const float* __res
   const float* src = w + i0 * 9;
   if (aligned_dev(src, 16)) {
     const int n4 = n >> 2;
-    for (int q = t; q < n4; q += kPatBlock) reinterpret_cast<float4*>(s_w)[q] = __ldg(reinterpret_cast<const float4*>(src) + q);
-    for (int q = 4 * n4 + t; q < n; q += kPatBlock) s_w[q] = __ldg(src + q);
+    for (int q = t; q < n4; q += kPatBlock) reinterpret_cast<float4*>(s_w)[q] = reinterpret_cast<const float4*>(src)[q];
+    for (int q = 4 * n4 + t; q < n; q += kPatBlock) s_w[q] = src[q];
   } else {
-    for (int q = t; q < n; q += kPatBlock) s_w[q] = __ldg(src + q);
+    for (int q = t; q < n; q += kPatBlock) s_w[q] = src[q];
   }
   __syncthreads();
   const bool in = i < FC;
