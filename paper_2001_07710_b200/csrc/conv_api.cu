@@ -8,11 +8,11 @@ bool conv_mma_f16_supported(int F, int C, int dtype, int N, int H, int W, int st
 int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, int64_t n_keep, const void* x, void* y,
                  int N, int H, int W, int stride, int act, unsigned long long wait_ns, int test_skip, cudaStream_t st);
 bool conv_mma_f32_supported(int F, int C, int dtype, int N, int H, int W, int stride);
-double conv_mma_f32_clocks(int F, int C, int N, int H, int W, int stride, int act);
+double conv_mma_f32_clocks(int F, int C, int N, int H, int W, int stride);
 int conv_mma_f32(const void* blob, int F, int C, const uint16_t* masks, int K, int64_t n_keep, const void* x, void* y,
                  int N, int H, int W, int stride, int act, unsigned long long wait_ns, int test_skip, cudaStream_t st);
 size_t conv_img_workspace(int F, int C, int dtype, int N, int H, int W, int stride);
-double conv_f32_img_clocks(int F, int C, const uint16_t* masks, int K, int64_t n_keep, int N, int H, int W, int act, int sms);
+double conv_f32_img_clocks(int F, int C, const uint16_t* masks, int K, int64_t n_keep, int N, int H, int W, int sms);
 int conv_f32_img(const void* blob, int F, int C, const uint16_t* masks, int K, int64_t n_keep,
                  const void* x, void* y, int N, int H, int W, int relu, void* workspace, cudaStream_t st);
 }
@@ -59,12 +59,13 @@ static int conv_mma(const void* blob, int F, int C, const uint16_t* masks, int K
 // Which kernels run an fp32 call with a workspace whose blob serves both: the ones with the smaller estimate.  Both sides
 // measured: 56x56x256 -> 256, batch 32, keep 1/8, eight patterns: multiply-adds 313 us, tensor cores 347 (six products
 // for 18 times the useful work); batch 1: 36 and 27 us (the multiply-add kernels' items do not fill the chip);
-// 28x28x256, batch 32, twelve patterns: 213 and 104 us.
-static bool prefer_img(int F, int C, const uint16_t* masks, int K, int64_t n_keep, int dtype, int N, int H, int W, int stride, int act) {
+// 28x28x256, batch 32, twelve patterns: 213 and 104 us.  The estimates are those of the plain convolution whatever follows it,
+// so that fused pooling has the sums of the two passes that it replaces (the two kernels' sums differ in their last bits).
+static bool prefer_img(int F, int C, const uint16_t* masks, int K, int64_t n_keep, int dtype, int N, int H, int W, int stride) {
   if (stride != 1 || !img_blocks(F, C, n_keep, dtype)) return false;     // stride 2 has a quarter of the positions there
   static thread_local DeviceSlot slots[kMaxDevices];
   DeviceSlot* dv = device_slot(slots);
-  return conv_f32_img_clocks(F, C, masks, K, n_keep, N, H, W, act, dv ? dv->sms : 148) < conv_mma_f32_clocks(F, C, N, H, W, stride, act);
+  return conv_f32_img_clocks(F, C, masks, K, n_keep, N, H, W, dv ? dv->sms : 148) < conv_mma_f32_clocks(F, C, N, H, W, stride);
 }
 
 extern "C" int pat_conv3x3(const void* blob, int F, int C, const uint16_t* masks, int K, int64_t n_keep,
@@ -97,7 +98,7 @@ extern "C" int pat_conv3x3_ws_act(const void* blob, int F, int C, const uint16_t
     if (!workspace || workspace_bytes < need)
       return set_error(PAT_ERR_WORKSPACE, "pat_conv3x3_ws: workspace has %zu bytes, needs %zu", workspace_bytes, need);
     if (!aligned(workspace, 256)) return set_error(PAT_ERR_ALIGN, "pat_conv3x3_ws: workspace must be 256-byte aligned");
-    if (prefer_img(F, C, masks, K, n_keep, dtype, N, H, W, stride, act))
+    if (prefer_img(F, C, masks, K, n_keep, dtype, N, H, W, stride))
       return conv_f32_img(blob, F, C, masks, K, n_keep, x, y, N, H, W, act, workspace, reinterpret_cast<cudaStream_t>(stream));
   }
   if (on_tensor_cores(F, C, dtype, N, H, W, stride)) return conv_mma(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride, act, stream);

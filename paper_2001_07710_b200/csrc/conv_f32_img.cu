@@ -641,7 +641,7 @@ size_t conv_img_workspace(int F, int C, int dtype, int N, int H, int W, int stri
 // Estimated clocks of a call: the stage-image pass at 5.5 TB/s, the results, then rounds x stages x what a stage takes - at least the copy of
 // its 72 KB (2100 clocks), plus its share of the kernels (23100 clocks when all are kept; libraries beyond the eight patterns
 // do not fit the instruction cache).  Fitted to 28x28 .. 224x224 layers at batch 8 and 32, keep 1/100 .. 1/2: within 10 %.
-double conv_f32_img_clocks(int F, int C, const uint16_t* masks, int K, int64_t n_keep, int N, int H, int W, int act, int sms) {
+double conv_f32_img_clocks(int F, int C, const uint16_t* masks, int K, int64_t n_keep, int N, int H, int W, int sms) {
   using namespace img32;
   Params p;
   if (!fill_geometry(p, F, C, N, H, W)) return 1e30;
@@ -652,7 +652,7 @@ double conv_f32_img_clocks(int F, int C, const uint16_t* masks, int K, int64_t n
   const double stage = 2100.0 + (eight ? 23100.0 : 79000.0) * keep;
   const double rounds = (double)((p.n_whole + grid - 1) / grid) + (p.parts > 1 ? 1.0 / p.parts : 0.0);
   const double pixels = (double)N * H * W;
-  return 3.2e-3 * pixels * C + 1.0e-3 * pixels * F / (act == 2 ? 4 : 1) + rounds * p.nct * stage + 6000.0 + (p.parts > 1 ? 20000.0 : 0.0);
+  return 3.2e-3 * pixels * C + 1.0e-3 * pixels * F + rounds * p.nct * stage + 6000.0 + (p.parts > 1 ? 20000.0 : 0.0);
 }
 
 int conv_f32_img(const void* blob, int F, int C, const uint16_t* masks, int K, int64_t n_keep,

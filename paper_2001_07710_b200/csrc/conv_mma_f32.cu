@@ -478,13 +478,12 @@ bool conv_mma_f32_supported(int F, int C, int dtype, int N, int H, int W, int st
 }
 
 // Estimated clocks of a call (13 % above the sum of its parts, as measured from 28x28 to 224x224 at batch 8 and 32).
-double conv_mma_f32_clocks(int F, int C, int N, int H, int W, int stride, int act) {
+double conv_mma_f32_clocks(int F, int C, int N, int H, int W, int stride) {
   using namespace tmma;
   const Device d = device();
   Geometry p;
   if (d.rc || !set_geometry(p, TILE, N, H, W, stride, 0)) return 1e30;
   const Split sp = choose_split(p.tiles, F, C, *d.at_once);
-  if (act == 2 && !set_geometry(p, TILE, N, H, W, stride, 2)) return 1e30;
   return 1.13 * split_clocks(sp, p.tiles, C, *d.at_once);
 }
 

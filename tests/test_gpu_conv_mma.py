@@ -131,3 +131,19 @@ def test_f32_ends_of_the_range(value):
     # one product per output: the three dropped products of parts are below 2^-25 of it, the sum of the six others is rounded in
     # fp32; parts below 2^-133 (the smallest bf16 step) are lost
     assert bool(((y.double() - ref).abs() <= 6 * STEP * ref.abs() + 2.0 ** -132 * float(w.abs().max())).all())
+
+
+# near the line between the two fp32 kernels, where estimates with and without pooling would fall on different sides of it
+@pytest.mark.parametrize("N,H,C", [(64, 56, 64), (2, 224, 64), (8, 224, 64), (4, 112, 128), (8, 56, 256)])
+def test_f32_fused_pooling_has_the_sums_of_the_two_passes(N, H, C):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(N + H + C)
+    w = torch.randn((C, C, 3, 3), generator=gen, device="cuda") * (2.0 / (9 * C)) ** 0.5
+    x = torch.randn((N, H, H, C), generator=gen, device="cuda").clamp_(min=0)
+    masks, n_keep = pc.pat_library_builtin(8), C * C // 8
+    pid, wm = pc.pat_project(w, masks, n_keep)
+    blob = pc.pat_pack(wm, pid, masks, n_keep, "f32")
+    fused = pc.pat_conv3x3(blob, C, C, masks, n_keep, "f32", x, 1, pool=True)
+    plain = pc.pat_conv3x3(blob, C, C, masks, n_keep, "f32", x, 1)
+    assert torch.equal(fused, pc.pat_relu_maxpool(plain, "f32", True))
+    assert torch.equal(pc.pat_conv3x3(blob, C, C, masks, n_keep, "f32", x, 1, relu=True), plain.clamp(min=0))
