@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
     const uint32_t st = sbase + OFF_ST;
     const int px = warp * 32 + lane;                   // position inside the tile
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const float floor_at = p.act != 0 ? 0.0f : -INFINITY;       // the rectifier
+    const float floor_at = p.act != 0 ? 0.0f : __uint_as_float(0x7FFFFFFFu);      // the rectifier: fmaxf(v, NaN) is v, a NaN too
     for (int item = unit; item < p.items && alive; item += n_units) {
       const int tg = p.d_groups.div(item), g = item - tg * p.groups;
       const int m0 = (CG == 2 ? 2 * tg + (int)rank : tg) * p.mstep;

@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
     const int px = (warp & 3) * 32 + lane;                     // position inside the tile
     const uint32_t st = sbase + OFF_ST;
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
-    const float floor_at = p.act != 0 ? 0.0f : -INFINITY;       // the rectifier
+    const float floor_at = p.act != 0 ? 0.0f : __uint_as_float(0x7FFFFFFFu);      // the rectifier: fmaxf(v, NaN) is v, a NaN too
     const int n_chunks = cb1 - cb0;
     int buf = 0;
     uint32_t pf = 0u;

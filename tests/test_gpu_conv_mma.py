@@ -147,3 +147,33 @@ def test_f32_fused_pooling_has_the_sums_of_the_two_passes(N, H, C):
     plain = pc.pat_conv3x3(blob, C, C, masks, n_keep, "f32", x, 1)
     assert torch.equal(fused, pc.pat_relu_maxpool(plain, "f32", True))
     assert torch.equal(pc.pat_conv3x3(blob, C, C, masks, n_keep, "f32", x, 1, relu=True), plain.clamp(min=0))
+
+
+# unsplit, channels cut among the CTAs of a cluster, several rounds with two accumulator sets, stride 2
+NOT_A_NUMBER = [(2, 56, 56, 64, 64, 8, 0.25, 1), (1, 14, 14, 512, 512, 8, 0.25, 1), (16, 28, 28, 64, 256, 8, 0.25, 1), (2, 15, 15, 48, 40, 8, 0.5, 2)]
+
+
+@pytest.mark.parametrize("dtype", ["f16", "f32"])
+@pytest.mark.parametrize("case", NOT_A_NUMBER, ids=lambda c: "-".join(str(v) for v in c))
+def test_a_result_that_is_not_a_number_stays_one(case, dtype):
+    """Outputs that a kept tap connects to a NaN are NaN without a rectifier; with one (and pooling) they are what
+    pat_relu_maxpool makes of that."""
+    N, H, W, C, F, K, keep, stride = case
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(C + F)
+    w = torch.randn((F, C, 3, 3), generator=gen, device="cuda") * (2.0 / (9 * C)) ** 0.5
+    x = torch.randn((N, H, W, C), generator=gen, device="cuda").clamp_(min=0).to(torch.float16 if dtype == "f16" else torch.float32)
+    masks, n_keep = pc.pat_library_builtin(K), int(F * C * keep)
+    pid, wm = pc.pat_project(w, masks, n_keep)
+    blob = pc.pat_pack(wm, pid, masks, n_keep, dtype)
+    x[N - 1, 6, 7, 3] = x[0, 0, 0, C - 1] = float("nan")
+    call = lambda **kw: pc.pat_conv3x3(blob, F, C, masks, n_keep, dtype, x, stride, **kw)
+    y = call()
+    kept = (pc.pat_unpack(blob, F, C, masks, n_keep, dtype) != 0).double()
+    touched = Fn.conv2d(torch.isnan(x).permute(0, 3, 1, 2).double(), kept, stride=stride, padding=1).permute(0, 2, 3, 1) > 0
+    assert int(touched.sum()) > F // 4
+    assert bool(torch.isnan(y[touched]).all())
+    assert torch.equal(call(relu=True), pc.pat_relu_maxpool(y, dtype, False))
+    if stride == 1:
+        assert torch.equal(call(pool=True), pc.pat_relu_maxpool(y, dtype, True))
+    assert pc.pat_query_status() == 0
