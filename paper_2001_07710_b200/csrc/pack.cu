@@ -176,6 +176,12 @@ template <typename T> __device__ inline T cvt_weight(float v);
 template <> __device__ inline float cvt_weight<float>(float v) { return v; }
 template <> __device__ inline __half cvt_weight<__half>(float v) { return __float2half_rn(v); }
 
+// The bf16 number next to v; a finite one that would round to infinity is cut off instead (its rest is a bf16 number too).
+__device__ inline __nv_bfloat16 finite_bf16(float v) {
+  const uint32_t b = __float_as_uint(v), r = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v));
+  return __ushort_as_bfloat16((unsigned short)((r & 0x7FFFu) == 0x7F80u ? b >> 16 : r));
+}
+
 // Two neighbouring values of the dense form: fp16, or fp32 as a sum of three bf16 numbers, each the rounded rest of those
 // before it.
 template <typename T> __device__ inline void dense_store(uint32_t* dst, size_t term, float v0, float v1);
@@ -185,7 +191,7 @@ template <> __device__ inline void dense_store<__half>(uint32_t* dst, size_t, fl
 template <> __device__ inline void dense_store<float>(uint32_t* dst, size_t term, float v0, float v1) {
 #pragma unroll
   for (int t = 0; t < kMmaTermsF32; ++t) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
+    const __nv_bfloat16 h0 = finite_bf16(v0), h1 = finite_bf16(v1);
     dst[t * term] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
     v0 -= __bfloat162float(h0);            // exact: the rest has fewer significant bits
     v1 -= __bfloat162float(h1);

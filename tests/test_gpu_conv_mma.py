@@ -177,3 +177,24 @@ def test_a_result_that_is_not_a_number_stays_one(case, dtype):
     if stride == 1:
         assert torch.equal(call(pool=True), pc.pat_relu_maxpool(y, dtype, True))
     assert pc.pat_query_status() == 0
+
+
+@pytest.mark.parametrize("value", [3.4028234e38, -3.4e38, 3.3961e38])
+def test_f32_largest_weights(value):
+    """Weights that bf16 would round to infinity."""
+    F, C, H = 16, 16, 9
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(6)
+    w = torch.randn((F, C, 3, 3), generator=gen, device="cuda")
+    w[::2, 5, 1, 1] = value                    # the centre belongs to every built-in mask
+    masks = pc.pat_library_builtin(4)
+    pid, wm = pc.pat_project(w, masks, F * C)
+    blob = pc.pat_pack(wm, pid, masks, F * C, "f32")
+    x = torch.zeros((1, H, H, C), device="cuda")
+    x[0, 2:7, 2:7, 5] = torch.rand((5, 5), generator=gen, device="cuda") * 2.0 ** -8
+    y = pc.pat_conv3x3(blob, F, C, masks, F * C, "f32", x, 1)
+    conv = lambda a, b: Fn.conv2d(a.permute(0, 3, 1, 2).double(), b.double(), padding=1).permute(0, 2, 3, 1)
+    ref, mag = conv(x, wm), conv(x.abs(), wm.abs())
+    assert bool(torch.isfinite(y).all())
+    # at most four products per output (one channel, four taps), each with three dropped products of parts below 2^-25 of it
+    assert bool(((y.double() - ref).abs() <= 6 * STEP * mag).all())
