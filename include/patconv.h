@@ -146,8 +146,9 @@ int pat_unpack(const void *blob, int F, int C, const uint16_t *masks, int K, int
  * Sums are fp32 and so are the products: fp16 inputs are multiplied exactly, fp32 inputs as three bf16 parts each, of whose
  * products those below 2^-25 of the result's terms are left out.  The result is stored in the blob's dtype (fp16: round to
  * nearest even).
- * F and C multiples of eight: the tensor cores run the dense form of the masked weights, zeros included, so inputs have to
- * be finite (an infinite input reaches every output in its 3 x 3 neighbourhood as a NaN, whatever the kernel's mask).
+ * F and C multiples of eight: the tensor cores run the dense form of the masked weights, zeros included.  An infinity or NaN
+ * reaches the outputs whose kept taps read it and no others all the same: results that the zeros would make NaN are formed
+ * again from the kept taps, which takes its time when there are many.
  *   blob     dev, written by pat_pack with the same (F, C, masks, K, n_keep, dtype)
  *   masks    host, the library the blob was packed with
  *   x        dev, NHWC [N][H][W][C], 16-byte aligned

@@ -45,7 +45,7 @@ struct BlobLayout {
   size_t dboff, dblk;                  // descriptor blocks (img_blocks; else empty)
   int nblk;                            // number of descriptor blocks = (F / 32) * (C / 8), or 0
   size_t dense;                        // masked weights in dense form for the tensor cores (see mma_weights)
-  size_t scratch;                      // pack-time temporaries: hist[F][K], count[F], inv[F], xinv[F], xbase[F], stage bits
+  size_t scratch;                      // pack-time temporaries: hist[F][K], count[F], inv[F] (kept, see inv_offset), xinv[F], xbase[F], stage bits
   size_t total;
   int nct;                             // number of 16-channel tiles = ceil(C / 16)
 };
@@ -93,6 +93,9 @@ __host__ __device__ inline BlobLayout blob_layout(int F, int C, int K, int64_t n
   L.total = o;
   return L;
 }
+
+// inv[F]: original filter -> its position in the canonical order.
+__host__ __device__ inline size_t inv_offset(const BlobLayout& L, int F, int K) { return L.scratch + sizeof(int32_t) * (size_t)F * ((size_t)K + 1); }
 
 // Library passed by value to kernels.
 struct MaskTable {

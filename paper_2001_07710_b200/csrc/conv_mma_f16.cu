@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
   const uint32_t received = sbase + 8u * (BARS - 3), go = sbase + 8u * (BARS - 2), drain = sbase + 8u * (BARS - 1);
   int& s_abort = *reinterpret_cast<int*>(smem + 8 * BARS);           // a wait has given up, or the blob was refused
   int& s_refused = *reinterpret_cast<int*>(smem + 8 * BARS + 4);
+  int& s_note = *reinterpret_cast<int*>(smem + 8 * BARS + 12);       // a result is not finite, see Note
   uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + 8 * BARS + 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
   if (threadIdx.x == 0) {
     s_abort = 0;
     s_refused = 0;
+    s_note = 0;
   }
   if (threadIdx.x == W_A * 32) prefetch_map(&maps.a);
   if (threadIdx.x == W_B * 32) prefetch_map(&maps.b);
@@ -296,7 +298,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
     const uint32_t st = sbase + OFF_ST;
     const int px = warp * 32 + lane;                   // position inside the tile
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const float floor_at = p.act != 0 ? 0.0f : __uint_as_float(0x7FFFFFFFu);      // the rectifier: fmaxf(v, NaN) is v, a NaN too
+    Note note;
+    const float floor_at = p.act != 0 ? 0.0f : -INFINITY;       // the rectifier
     for (int item = unit; item < p.items && alive; item += n_units) {
       const int tg = p.d_groups.div(item), g = item - tg * p.groups;
       const int m0 = (CG == 2 ? 2 * tg + (int)rank : tg) * p.mstep;
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
           }
         }
         alive = close_exchange(p, received, alive, abort_flag);
-        if (alive) add_parts<false, TILE, 1>(p, sbase, item, rank);
+        if (alive) add_parts<false, TILE, 1>(p, sbase, item, rank, note);
         break;
       }
       for (int c0 = 0; c0 < p.BN; c0 += CCOLS) {
@@ -353,13 +356,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
           if (q * 16 >= nc) break;
           float f[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) f[i] = fmaxf(__uint_as_float(v[q][i]), floor_at);
+          for (int i = 0; i < 16; ++i) f[i] = max_nan(__uint_as_float(v[q][i]), floor_at);
           stage_results<false>(row, sw, q, f);
         }
-        store_results<false, 1>(p, st, g, c0, nc, pixel, m0, warp, lane);
+        store_results<false, 1>(p, st, g, c0, nc, pixel, m0, warp, lane, note);
       }
       if (++buf == n_acc) { buf = 0; pf ^= 1u; }
     }
+    if (note.taken()) s_note = 1;
   }
   if (!alive && !s_refused) atomicExch(p.status, PAT_ERR_TIMEOUT);
   __syncwarp();
@@ -384,6 +388,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
   if (failed && p.parts > 1) give_time();              // what the others had sent by then
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == W_MMA) free_columns<CG>(tmem);
+  if (s_note && !failed) {
+    const bool whole = CG == 2 || p.parts == 1;
+    renew_results<false, CG>(p, unit, n_units, CG == 2 ? (int)rank : 0, whole ? 0 : first_column<false>(p, (int)rank),
+                             whole ? p.BN : first_column<false>(p, (int)rank + 1));
+  }
 }
 
 // How the work is cut: pairs of CTAs over large problems; single CTAs, the channels cut among the CTAs of a cluster, over
@@ -450,7 +459,7 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   if (act == 2 && !set_geometry(p, TILE, N, H, W, stride, 2)) return set_error(PAT_ERR_SHAPE, "pat_conv3x3: too many tiles");
   p.act = act;
   p.y = y;
-  p.hdr = reinterpret_cast<const BlobHeader*>(b);
+  set_packed(p, x, blob, L, F, K);
   p.status = status_word();
   if (!p.status) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cannot resolve the status word");
   p.F = F; p.C = C; p.K = K; p.dtype = PAT_F16; p.n_keep = n_keep;

@@ -43,7 +43,6 @@ constexpr int BUF_COLS = 256;              // tensor memory: two buffers of 128 
 
 struct alignas(64) Maps { CUtensorMap b; };
 struct Params : Geometry {
-  const float* x;
   int a_rows, a_slots;       // activations: rows of a part of a stage, ring slots
   uint32_t a_bytes;          // bytes of a slot (three parts)
 };
@@ -86,6 +85,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
   const uint32_t received = sbase + 8u * (BARS - 3), go = sbase + 8u * (BARS - 2), drain = sbase + 8u * (BARS - 1);
   int& s_abort = *reinterpret_cast<int*>(smem + 8 * BARS);           // a wait has given up, or the blob was refused
   int& s_refused = *reinterpret_cast<int*>(smem + 8 * BARS + 4);
+  int& s_note = *reinterpret_cast<int*>(smem + 8 * BARS + 12);       // a result is not finite, see Note
   uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + 8 * BARS + 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank(), side = rank % CG, pair = rank - side, part = rank / CG;
@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
   if (threadIdx.x == 0) {
     s_abort = 0;
     s_refused = 0;
+    s_note = 0;
   }
   if (threadIdx.x == W_B * 32) prefetch_map(&maps.b);
   if (threadIdx.x < BARS) {                // a barrier each: 30 of them in a row by one thread showed in the launch
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
             v[j][1] = v[j][0];
             if (((valid >> (4 * j + pl)) & 1u) && c < p.C) {
               // not through the read-only path: the kernel that writes x may still run when this block starts
-              const float4* src = reinterpret_cast<const float4*>(p.x + (size_t)(base[j] + shift) * p.C + c);
+              const float4* src = reinterpret_cast<const float4*>(static_cast<const float*>(p.x) + (size_t)(base[j] + shift) * p.C + c);
               v[j][0] = src[0];
               v[j][1] = src[1];
             }
@@ -323,7 +324,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
     const int px = (warp & 3) * 32 + lane;                     // position inside the tile
     const uint32_t st = sbase + OFF_ST;
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
-    const float floor_at = p.act != 0 ? 0.0f : __uint_as_float(0x7FFFFFFFu);      // the rectifier: fmaxf(v, NaN) is v, a NaN too
+    Note note;
+    const float floor_at = p.act != 0 ? 0.0f : -INFINITY;       // the rectifier
     const int n_chunks = cb1 - cb0;
     int buf = 0;
     uint32_t pf = 0u;
@@ -375,7 +377,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
           for (int q = 0; q < 4; ++q)
             if (q * 16 < half) send_part<true, TILE, CG>(p, sbase, received, rank, col0 + q * 16, px, pixel >= 0, acc[q]);
         alive = close_exchange(p, received, alive, abort_flag);
-        if (alive) add_parts<true, TILE, CG>(p, sbase, item, rank);
+        if (alive) add_parts<true, TILE, CG>(p, sbase, item, rank, note);
         break;
       }
       const uint32_t row = st + (uint32_t)(warp * 32 + lane) * 128u, sw = (uint32_t)(lane & 7);
@@ -387,12 +389,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
             if ((2 * h + q) * 16 < half) {
               float f[16];
 #pragma unroll
-              for (int i = 0; i < 16; ++i) f[i] = fmaxf(acc[2 * h + q][i], floor_at);
+              for (int i = 0; i < 16; ++i) f[i] = max_nan(acc[2 * h + q][i], floor_at);
               stage_results<true>(row, sw, q, f);
             }
-          store_results<true, 2>(p, st, g, col0 + h * 32, min(32, half - h * 32), pixel, m0, warp, lane);
+          store_results<true, 2>(p, st, g, col0 + h * 32, min(32, half - h * 32), pixel, m0, warp, lane, note);
         }
     }
+    if (note.taken()) s_note = 1;
   }
   if (!alive && !s_refused) atomicExch(p.status, PAT_ERR_TIMEOUT);
   __syncwarp();
@@ -417,6 +420,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
   if (failed && p.parts > 1) give_time();              // what the others had sent by then
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == W_MMA) free_columns<CG>(tmem);
+  if (s_note && !failed) {
+    const bool whole = p.parts == 1;
+    renew_results<true, CG>(p, unit, n_units, (int)side, whole ? 0 : first_column<true>(p, (int)part), whole ? p.BN : first_column<true>(p, (int)part + 1));
+  }
 }
 
 // How the work is cut (pairs or single CTAs, filters per group, channel pieces): the choice with the smallest estimated time.
@@ -499,9 +506,8 @@ int conv_mma_f32(const void* blob, int F, int C, const uint16_t* masks, int K, i
   Split sp = choose_split(p.tiles, F, C, *d.at_once);           // the same for every `act`: the same sums
   if (act == 2 && !set_geometry(p, TILE, N, H, W, stride, 2)) return set_error(PAT_ERR_SHAPE, "pat_conv3x3: too many tiles");
   p.act = act;
-  p.x = static_cast<const float*>(x);
   p.y = y;
-  p.hdr = reinterpret_cast<const BlobHeader*>(b);
+  set_packed(p, x, blob, L, F, K);
   p.status = status_word();
   if (!p.status) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cannot resolve the status word");
   p.F = F; p.C = C; p.K = K; p.dtype = PAT_F32; p.n_keep = n_keep;

@@ -34,8 +34,12 @@ constexpr uint32_t TMEM_COLS = 512;
 
 // What the kernels' parameter blocks have in common.
 struct Geometry {
+  const void* x;
   void* y;
   const BlobHeader* hdr;
+  const int32_t *inv, *pptr; // the packed kernels in canonical order, see kept_taps
+  const uint16_t* chan;
+  const void* w4;
   int* status;
   int N, H, W, F, C, K, dtype;
   long long n_keep;
@@ -217,6 +221,12 @@ __device__ __forceinline__ int pixel_of(const Geometry& p, int m, int& y, int& x
 }
 
 // ------------------------------------------------------------------------------------------ results
+// The larger one, NaN if one of them is.  (fmaxf and __hmax2 give the other one.)
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  return m;
+}
 template <bool F32>
 __device__ __forceinline__ uint32_t max1(uint32_t a, uint32_t b) {
   if constexpr (F32) return __float_as_uint(fmaxf(__uint_as_float(a), __uint_as_float(b)));
@@ -228,11 +238,124 @@ __device__ __forceinline__ uint4 max4(const uint4& a, const uint4& b) {
   return make_uint4(max1<F32>(a.x, b.x), max1<F32>(a.y, b.y), max1<F32>(a.z, b.z), max1<F32>(a.w, b.w));
 }
 
+// Infinities and NaN.  The dense form multiplies an input by the zeros of removed taps and kernels too, and zero times
+// infinity is no number; of an infinity the fp32 kernel's three parts are infinity, NaN and NaN.  So a sum that is not a number
+// may only say that something in its neighbourhood is not finite, and is formed again from the kept taps alone.  (A sum that
+// is a number needs nothing: an infinity that it read met a kept weight.)  The epilogue stores such a sum as NaN, with a
+// rectifier too, and takes a note; a block that has taken one goes over its results again at the end, when nothing waits
+// for it.  With pooling the numbers of a window are stored, and which of its sums were none is told by the inputs and weights
+// that they read.  (Forming them in the epilogue itself, out of line, took 0.6 us of an 8.7 us launch in fp16 and 2 of 10 in
+// fp32: a call inside its loops costs registers whether it is taken or not.)
+struct Note {                              // zero as long as all values seen were finite, then NaN
+  float2 t = {0.0f, 0.0f};
+  template <bool F32>
+  __device__ __forceinline__ void see(const uint4& v) {
+    if constexpr (F32) {
+      t.x = fmaf(__uint_as_float(v.x), 0.0f, t.x);
+      t.y = fmaf(__uint_as_float(v.y), 0.0f, t.y);
+      t.x = fmaf(__uint_as_float(v.z), 0.0f, t.x);
+      t.y = fmaf(__uint_as_float(v.w), 0.0f, t.y);
+    } else {
+      const __half2 z = __float2half2_rn(0.0f);
+      const __half2* h = reinterpret_cast<const __half2*>(&v);
+      __half2 s = *reinterpret_cast<__half2*>(&t.x);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s = __hfma2(h[i], z, s);
+      t.x = *reinterpret_cast<float*>(&s);
+    }
+  }
+  // (floats or pairs of halves, each of either sign's zero or NaN)
+  __device__ __forceinline__ bool taken() const { return ((__float_as_uint(t.x) | __float_as_uint(t.y)) & 0x7FFF7FFFu) != 0u; }
+};
+template <bool F32>
+__device__ __forceinline__ float stored(const void* a, size_t i) {
+  if constexpr (F32) return static_cast<const float*>(a)[i];
+  else return __half2float(static_cast<const __half*>(a)[i]);
+}
+// The sum over the kept taps of filter f for output (n, y, x), in fp32: what the packed weights say.
+template <bool F32>
+__device__ __noinline__ float kept_taps(const Geometry& p, int f, int n, int y, int x) {
+  const int32_t* pp = p.pptr + (size_t)p.inv[f] * (p.K + 1);
+  const int y0 = y * p.stride - 1, x0 = x * p.stride - 1;
+  float sum = 0.0f;
+  for (int j = 0; j < p.K; ++j)
+    for (int k = pp[j]; k < pp[j + 1]; ++k) {
+      const int c = p.chan[k];
+      unsigned m = p.masks[j];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {                    // ascending bit order
+        const int b = __ffs(m) - 1, yy = y0 + b / 3, xx = x0 + b % 3;
+        m &= m - 1u;
+        if (yy >= 0 && yy < p.H && xx >= 0 && xx < p.W)
+          sum = fmaf(stored<F32>(p.x, (((size_t)n * p.H + yy) * p.W + xx) * p.C + c), stored<F32>(p.w4, (size_t)k * 4 + t), sum);
+      }
+    }
+  return sum;
+}
+template <bool F32>
+__device__ __forceinline__ void store_one(const Geometry& p, size_t at, float v) {
+  if constexpr (F32) static_cast<float*>(p.y)[at] = v;
+  else static_cast<__half*>(p.y)[at] = __float2half_rn(v);
+}
+// The results that this block has stored - columns c_begin to c_end of its items - gone over by all its warps.
+template <bool F32, int CG>
+__device__ __noinline__ void renew_results(const Geometry& p, int unit, int n_units, int side, int c_begin, int c_end) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
+  const int hw = p.Ws >> 1, n_out = p.act == 2 ? (p.d_P.div(p.mstep) >> 1) * hw : p.mstep;
+  for (int item = unit; item < p.items; item += n_units) {
+    const int tg = p.d_groups.div(item), g = item - tg * p.groups, m0 = (CG * tg + side) * p.mstep;
+    const int f0 = g * p.BN + c_begin, f1 = min(g * p.BN + c_end, p.F);
+    unsigned odd_filter = 0u;                          // bit j: filter f0 + lane + 32 j has a weight that is not finite
+    if (p.act == 2)
+      for (int f = f0 + lane, j = 0; f < f1; f += 32, ++j) {
+        const int32_t* pp = p.pptr + (size_t)p.inv[f] * (p.K + 1);
+        for (size_t i = (size_t)pp[0] * 4; i < (size_t)pp[p.K] * 4; ++i)
+          if (!isfinite(stored<F32>(p.w4, i))) odd_filter |= 1u << j;
+      }
+    for (int t = warp; t < n_out; t += warps) {        // a warp per output pixel
+      int yy, xx, nn;
+      if (p.act != 2) {
+        const int pixel = pixel_of(p, m0 + t, yy, xx, nn);
+        if (pixel < 0) continue;
+        for (int f = f0 + lane; f < f1; f += 32) {
+          const size_t at = (size_t)pixel * p.F + f;
+          const float old = stored<F32>(p.y, at);
+          if (old == old) continue;
+          const float v = kept_taps<F32>(p, f, nn, yy, xx);
+          store_one<F32>(p, at, p.act ? fmaxf(v, 0.0f) : v);       // (what pat_relu_maxpool makes of a NaN)
+        }
+        continue;
+      }
+      const int jj = t / hw;
+      if (pixel_of(p, m0 + 2 * jj * p.P + 2 * (t - jj * hw), yy, xx, nn) < 0) continue;
+      unsigned odd = 0u;                               // bit k: the window's k-th sum has read an input that is not finite
+      for (int k = 0; k < 4; ++k) {
+        bool any = false;
+        for (int b = 0; b < 9; ++b) {
+          const int y = yy + (k >> 1) + b / 3 - 1, x = xx + (k & 1) + b % 3 - 1;
+          if (y < 0 || y >= p.H || x < 0 || x >= p.W) continue;
+          for (int c = lane; c < p.C; c += 32) any = any || !isfinite(stored<F32>(p.x, (((size_t)nn * p.H + y) * p.W + x) * p.C + c));
+        }
+        if (__any_sync(0xFFFFFFFFu, any)) odd |= 1u << k;
+      }
+      for (int f = f0 + lane, j = 0; f < f1; f += 32, ++j) {
+        const unsigned again = (odd_filter >> j) & 1u ? 15u : odd;
+        if (!again) continue;
+        const size_t at = (((size_t)nn * (p.Ho >> 1) + (yy >> 1)) * (p.Wo >> 1) + (xx >> 1)) * p.F + f;
+        float v = fmaxf(stored<F32>(p.y, at), 0.0f);
+        for (int k = 0; k < 4; ++k)
+          if ((again >> k) & 1u) v = fmaxf(v, kept_taps<F32>(p, f, nn, yy + (k >> 1), xx + (k & 1)));
+        store_one<F32>(p, at, v);
+      }
+    }
+  }
+}
+
 // One pass of the epilogue: the results of up to 64 fp16 / 32 fp32 columns lie in the staging, 128 bytes per position
 // (16-byte chunks swizzled by the position's low bits), and leave as runs of 128 bytes of NHWC output.  HALVES = 2: warps
 // 4-7 hold other columns of the same 128 positions (in staging rows 128-255) instead of 128 more positions.
 template <bool F32, int HALVES>
-__device__ __forceinline__ void store_results(const Geometry& p, uint32_t st, int g, int c0, int nc, int pixel, int m0, int warp, int lane) {
+__device__ __forceinline__ void store_results(const Geometry& p, uint32_t st, int g, int c0, int nc, int pixel, int m0, int warp, int lane, Note& note) {
   constexpr int PER = F32 ? 4 : 8;                     // values per 16-byte chunk
   const int q = lane & 7, f = g * p.BN + c0 + q * PER;
   const bool mine = q * PER < nc && f < p.F;
@@ -248,7 +371,10 @@ __device__ __forceinline__ void store_results(const Geometry& p, uint32_t st, in
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
       const int px = __shfl_sync(0xFFFFFFFFu, pixel, it * 4 + (lane >> 3));
-      if (px >= 0 && mine) *reinterpret_cast<uint4*>(y + ((size_t)px * p.F + f) * (F32 ? 4 : 2)) = v[it];
+      if (px >= 0 && mine) {
+        note.see<F32>(v[it]);
+        *reinterpret_cast<uint4*>(y + ((size_t)px * p.F + f) * (F32 ? 4 : 2)) = v[it];
+      }
     }
     __syncwarp();
     return;
@@ -270,6 +396,9 @@ __device__ __forceinline__ void store_results(const Geometry& p, uint32_t st, in
       tile::lds128(st + (uint32_t)r * 128u + (uint32_t)((q ^ (r & 7)) << 4), w[k].x, w[k].y, w[k].z, w[k].w);
     }
     const uint4 m = max4<F32>(max4<F32>(w[0], w[1]), max4<F32>(w[2], w[3]));
+    if (keep)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) note.see<F32>(w[k]);
     if (keep) *reinterpret_cast<uint4*>(y + ((((size_t)n * (p.Ho >> 1) + (yy >> 1)) * (p.Wo >> 1) + (xx >> 1)) * p.F + f) * (F32 ? 4 : 2)) = m;
   }
   asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
@@ -324,7 +453,7 @@ __device__ __forceinline__ void send_part(const Geometry& p, uint32_t sbase, uin
 }
 // This CTA's share, by the epilogue's warps, in the order of the channels.
 template <bool F32, int T, int CG>
-__device__ __forceinline__ void add_parts(const Geometry& p, uint32_t sbase, int item, uint32_t rank) {
+__device__ __forceinline__ void add_parts(const Geometry& p, uint32_t sbase, int item, uint32_t rank, Note& note) {
   constexpr int PER = kPer<F32>, Q = PER / 4, THREADS = EPI_WARPS * 32;
   const int side = (int)rank % CG, part = (int)rank / CG;
   const int tg = p.d_groups.div(item), g = item - tg * p.groups, m0 = (CG * tg + side) * p.mstep;
@@ -371,15 +500,21 @@ __device__ __forceinline__ void add_parts(const Geometry& p, uint32_t sbase, int
           for (int i = 0; i < 4; ++i) v[4 * j + i] += __uint_as_float(w[q][i]);
         }
       }
+      if (pool)
+#pragma unroll
+        for (int j = 0; j < PER; j += 4)
+          note.see<true>(make_uint4(__float_as_uint(v[j]), __float_as_uint(v[j + 1]), __float_as_uint(v[j + 2]), __float_as_uint(v[j + 3])));
 #pragma unroll
       for (int j = 0; j < PER; ++j) s[j] = k == 0 ? v[j] : fmaxf(s[j], v[j]);
     }
     if (p.act)
 #pragma unroll
-      for (int j = 0; j < PER; ++j) s[j] = fmaxf(s[j], 0.0f);
+      for (int j = 0; j < PER; ++j) s[j] = pool ? fmaxf(s[j], 0.0f) : max_nan(s[j], 0.0f);
     uint4 r;
     if constexpr (F32) r = make_uint4(__float_as_uint(s[0]), __float_as_uint(s[1]), __float_as_uint(s[2]), __float_as_uint(s[3]));
     else r = make_uint4(pack_f16(s[0], s[1]), pack_f16(s[2], s[3]), pack_f16(s[4], s[5]), pack_f16(s[6], s[7]));
+    if (!pool) note.see<true>(make_uint4(__float_as_uint(s[0]), __float_as_uint(s[1]), __float_as_uint(s[2]), __float_as_uint(s[3])));
+    if (!pool && PER == 8) note.see<true>(make_uint4(__float_as_uint(s[PER - 4]), __float_as_uint(s[PER - 3]), __float_as_uint(s[PER - 2]), __float_as_uint(s[PER - 1])));
     *reinterpret_cast<uint4*>(y + (out * p.F + f) * (F32 ? 4 : 2)) = r;
   }
 }
@@ -443,6 +578,17 @@ inline int set_exchange(Geometry& p, int per, int smem_bytes, int ring_at, int r
   if ((int)p.recv - ring_at >= ring_needs) return std::min(ring_bytes, (int)p.recv - ring_at);
   p.handshake = 1;
   return ring_bytes;
+}
+
+// Where the packed kernels are (see kept_taps).
+inline void set_packed(Geometry& p, const void* x, const void* blob, const BlobLayout& L, int F, int K) {
+  const char* b = static_cast<const char*>(blob);
+  p.x = x;
+  p.hdr = reinterpret_cast<const BlobHeader*>(b);
+  p.inv = reinterpret_cast<const int32_t*>(b + inv_offset(L, F, K));
+  p.pptr = reinterpret_cast<const int32_t*>(b + L.pptr);
+  p.chan = reinterpret_cast<const uint16_t*>(b + L.chan);
+  p.w4 = b + L.w4;
 }
 
 // Positions, tiles and their input rows (see the head of the file).  False: more than an int counts.

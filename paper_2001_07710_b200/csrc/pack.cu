@@ -48,7 +48,7 @@ __host__ __device__ inline BlobPtrs blob_ptrs(void* blob, const BlobLayout& L, i
   p.dense = L.scratch > L.dense ? reinterpret_cast<unsigned short*>(b + L.dense) : nullptr;
   p.hist = reinterpret_cast<int32_t*>(b + L.scratch);
   p.cnt = p.hist + (size_t)F * K;
-  p.inv = p.cnt + F;
+  p.inv = reinterpret_cast<int32_t*>(b + inv_offset(L, F, K));
   p.xinv = p.inv + F;
   p.xbase = p.xinv + F;
   p.stages = reinterpret_cast<uint32_t*>(p.xbase + F);

@@ -198,3 +198,40 @@ def test_f32_largest_weights(value):
     assert bool(torch.isfinite(y).all())
     # at most four products per output (one channel, four taps), each with three dropped products of parts below 2^-25 of it
     assert bool(((y.double() - ref).abs() <= 6 * STEP * mag).all())
+
+
+@pytest.mark.parametrize("dtype", ["f16", "f32"])
+@pytest.mark.parametrize("case", NOT_A_NUMBER + [(1, 10, 130, 72, 136, 12, 0.5, 1)], ids=lambda c: "-".join(str(v) for v in c))
+def test_an_infinite_input_reaches_only_the_kept_taps(case, dtype):
+    """The tensor cores run removed taps as zeros: an infinity or NaN of the input must not come through them."""
+    N, H, W, C, F, K, keep, stride = case
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(C * F)
+    w = torch.randn((F, C, 3, 3), generator=gen, device="cuda") * (2.0 / (9 * C)) ** 0.5
+    x = torch.randn((N, H, W, C), generator=gen, device="cuda").clamp_(min=0).to(torch.float16 if dtype == "f16" else torch.float32)
+    masks, n_keep = pc.pat_library_builtin(K), int(F * C * keep)
+    pid, wm = pc.pat_project(w, masks, n_keep)
+    blob = pc.pat_pack(wm, pid, masks, n_keep, dtype)
+    x[N - 1, 6, 7, 3] = x[0, 0, 0, C - 1] = x[0, H - 1, W - 1, 0] = x[0, 8, 4, 5] = float("inf")
+    x[0, 9, 5, 20] = -float("inf")             # with its neighbour of the other sign: some outputs read both
+    x[N - 1, 3, W - 1, 9] = float("nan")
+    call = lambda **kw: pc.pat_conv3x3(blob, F, C, masks, n_keep, dtype, x, stride, **kw)
+    y = call()
+    wd = pc.pat_unpack(blob, F, C, masks, n_keep, dtype).double()
+    conv = lambda a, b: Fn.conv2d(a.permute(0, 3, 1, 2).double(), b.double(), stride=stride, padding=1).permute(0, 2, 3, 1)
+    finite = torch.where(torch.isfinite(x), x, torch.zeros_like(x))
+    up = conv(torch.isposinf(x), wd > 0) + conv(torch.isneginf(x), wd < 0) > 0.5
+    down = conv(torch.isposinf(x), wd < 0) + conv(torch.isneginf(x), wd > 0) > 0.5
+    none = (conv(torch.isnan(x), wd != 0) > 0.5) | (up & down)
+    up, down = up & ~none, down & ~none
+    assert int(none.sum()) and int(up.sum()) and int(down.sum())
+    assert torch.equal(torch.isnan(y), none) and torch.equal(torch.isposinf(y), up) and torch.equal(torch.isneginf(y), down)
+    ref, mag = conv(finite, wd), conv(finite.abs(), wd.abs())
+    bound = 4 * C * STEP * mag + (F16_ROUND * ref.abs() + 2.0 ** -25 if dtype == "f16" else 0.0)
+    assert bool(((y.double() - ref).abs() <= bound)[~(none | up | down)].all())
+    assert torch.equal(call(relu=True), pc.pat_relu_maxpool(y, dtype, False))
+    if stride == 1 and H % 2 == 0 and W % 2 == 0 and pc.pat_conv3x3_workspace(F, C, dtype, N, H, W, 1):
+        assert torch.equal(call(pool=True), pc.pat_relu_maxpool(y, dtype, True))
+    assert pc.pat_query_status() == 0
+    x.fill_(float("nan"))                      # every output is formed again
+    assert torch.equal(torch.isnan(call()), conv(torch.ones_like(x), wd != 0) > 0.5) and pc.pat_query_status() == 0
