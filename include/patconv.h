@@ -144,7 +144,8 @@ int pat_unpack(const void *blob, int F, int C, const uint16_t *masks, int K, int
  *   Y[n][y][x][f] = sum over kept kernels (f,c) and their four taps (r,s) of
  *                   w[f][c][r][s] * X[n][y*stride + r - 1][x*stride + s - 1][c]
  * Sums are fp32 and so are the products: fp16 inputs are multiplied exactly, fp32 inputs as three bf16 parts each, of whose
- * products those below 2^-25 of the result's terms are left out.  The result is stored in the blob's dtype (fp16: round to
+ * products those below 2^-25 of the result's terms are left out.  The tensor cores' own sums drop what does not fit their last
+ * bit; they run over 512 channels in fp16 and 32 in fp32 at most and are added up rounded to nearest.  The result is stored in the blob's dtype (fp16: round to
  * nearest even).
  * F and C multiples of eight: the tensor cores run the dense form of the masked weights, zeros included.  An infinity or NaN
  * reaches the outputs whose kept taps read it and no others all the same: results that the zeros would make NaN are formed

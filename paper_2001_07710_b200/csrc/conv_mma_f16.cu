@@ -20,6 +20,11 @@
 // positions.  CG = 1 (small problems): one CTA per 256 positions and up to 128 filters, the input channels cut into
 // `parts` pieces that run on the CTAs of a cluster and are added up through distributed shared memory in a fixed order.
 //
+// Accuracy.  Products are exact in the tensor core's fp32 sums, but those drop what does not fit their last bit, about 2^-24.5
+// of the running sum a step, so long sums drift towards zero.  They are no longer than CHUNK channels (288 steps; positive
+// data: 1.2e-5 low, against 2^-11 of rounding the result); further chunks are added up, rounded to nearest, in columns of
+// tensor memory of their own, which halves the filters that a pair takes.
+//
 // Roles: warps 0-7 epilogue (tensor memory -> fp32 -> rectifier -> fp16 -> shared memory -> coalesced stores), warp 8
 // copies activations, warp 9 weights, warp 10 issues the multiply-adds (in the even CTA of a pair).  Every wait is
 // bounded; tensor memory is released on every path.
@@ -33,6 +38,7 @@ constexpr int TILE = 256;                   // positions per CTA
 constexpr int KB = 64;                      // channels per stage (128 bytes)
 constexpr int W_A = 8, W_B = 9, W_MMA = 10, NWARPS = 12, NTHREADS = NWARPS * 32;
 constexpr int MAX_A = 4, MAX_B = 8;             // ring slots
+constexpr int CHUNK = 8;                        // channel blocks in one sum of the tensor core
 constexpr int ST_BYTES = TILE * 128;            // epilogue staging: 128 bytes per position
 constexpr int OFF_RING = 1024, RING_BYTES = 198656, OFF_ST = OFF_RING + RING_BYTES, SMEM_BYTES = OFF_ST + ST_BYTES;
 static_assert(SMEM_BYTES <= 232448 && OFF_ST % 1024 == 0, "shared memory budget of one SM");
@@ -46,7 +52,8 @@ struct Params : Geometry {
   int resident;              // the weights of the only group stay in shared memory
 };
 
-template <int CG>
+// LONG: more than CHUNK channel blocks.  (A variant of its own: in the common one the branches took 1 % of VGG-16.)
+template <int CG, bool LONG>
 __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_constant__ Maps maps, const __grid_constant__ Params p) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sbase = smem_u32(smem);
@@ -96,7 +103,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
   const uint32_t tmem = s_tmem;
   const uint32_t ring_b = sbase + OFF_RING + (uint32_t)p.a_slots * p.a_bytes;
 
-  const int n_acc = 2 * 2 * p.BN <= (int)TMEM_COLS ? 2 : 1;      // accumulator sets
+  // accumulator sets, beside the columns of the sums over several chunks
+  const int sum_cols = LONG ? 2 * p.BN : 0, n_acc = 2 * 2 * p.BN + sum_cols <= (int)TMEM_COLS ? 2 : 1;
   // CG = 2: a pair walks over the items; CG = 1: a cluster of `parts` CTAs has one item, or single CTAs walk
   const int unit = CG == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x / p.parts;
   const int n_units = CG == 2 ? (int)(gridDim.x >> 1) : (int)gridDim.x / p.parts;
@@ -221,10 +229,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
       const uint32_t a_step = p.a_bytes >> 4, b_step = p.b_bytes >> 4;
       for (int item = unit; item < p.items && alive; item += n_units) {
         if (!wait_warp(acc_empty(buf), pe, abort_flag, p.wait_ns)) { alive = false; break; }
-        const uint32_t d0 = utmem + (uint32_t)(buf * 2 * p.BN), d1 = d0 + (uint32_t)p.BN;
+        uint32_t d0 = utmem + (uint32_t)(buf * 2 * p.BN), d1 = d0 + (uint32_t)p.BN;
         uint32_t acc = 0u;
         uint32_t b_res = ringb_lo;
-        for (int cb = cb0; cb < cb1 && alive; ++cb) {
+        for (int cb = cb0, chunk_end = cb0 + CHUNK; cb < cb1 && alive; ++cb) {
+          if (LONG && cb == chunk_end) {       // on with the next set
+            chunk_end += CHUNK;
+            if (el) commit<CG>(acc_full(buf), 0u);
+            __syncwarp();
+            if (++buf == n_acc) { buf = 0; pe ^= 1u; }
+            if (!wait_warp(acc_empty(buf), pe, abort_flag, p.wait_ns)) { alive = false; break; }
+            d0 = utmem + (uint32_t)(buf * 2 * p.BN);
+            d1 = d0 + (uint32_t)p.BN;
+            acc = 0u;
+          }
           const int ks = cb + 1 == p.ncb ? p.ks_last : KB / 16;
           for (int pl = 0; pl < p.planes && alive; ++pl) {
             const int py = pl >> 1, px = pl & 1, nr = axis_taps(p.stride, py), nc = axis_taps(p.stride, px);
@@ -305,7 +323,32 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
       const int m0 = (CG == 2 ? 2 * tg + (int)rank : tg) * p.mstep;
       int yy, xx, nn;
       const int pixel = pixel_of(p, m0 + px, yy, xx, nn);
-      alive = mbar_wait<20>(acc_full(buf), pf, abort_flag, p.wait_ns);
+      // the chunks but the last
+      const uint32_t scol = lane_base + (uint32_t)(n_acc * 2 * p.BN + (warp >> 2) * p.BN);
+      bool summed = false;
+      for (int cb = cb0 + CHUNK; LONG && cb < cb1; cb += CHUNK) {
+        alive = __all_sync(0xFFFFFFFFu, mbar_wait<20>(acc_full(buf), pf, abort_flag, p.wait_ns)) != 0;
+        if (!alive) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t tcol = lane_base + (uint32_t)(buf * 2 * p.BN + (warp >> 2) * p.BN);
+        for (int c = 0; c < p.BN; c += 16) {
+          uint32_t v[16];
+          tmem_load16(tcol + (uint32_t)c, v);
+          tile::tmem_wait_ld();
+          if (summed) tmem_add16(scol + (uint32_t)c, v);
+          tmem_store16(scol + (uint32_t)c, v);
+        }
+        tile::tmem_wait_st();
+        summed = true;
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          if (CG == 2) arrive_remote(map_to_rank(acc_empty(buf), 0));
+          else mbar_arrive(acc_empty(buf));
+        }
+        if (++buf == n_acc) { buf = 0; pf ^= 1u; }
+      }
+      alive = alive && mbar_wait<20>(acc_full(buf), pf, abort_flag, p.wait_ns);
       if (p.act == 2 || p.parts > 1) alive = all_epilogue_warps(alive);       // they meet at barriers below: all go on or none
       if (!__all_sync(0xFFFFFFFFu, alive)) { alive = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -322,6 +365,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
             uint32_t v[16];
             tmem_load16(tcol + (uint32_t)c, v);
             tile::tmem_wait_ld();
+            if (LONG && summed) tmem_add16(scol + (uint32_t)c, v);
             float f[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
@@ -354,6 +398,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
 #pragma unroll
         for (int q = 0; q < CCOLS / 16; ++q) {
           if (q * 16 >= nc) break;
+          if (LONG && summed) tmem_add16(scol + (uint32_t)(c0 + q * 16), v[q]);
           float f[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) f[i] = max_nan(__uint_as_float(v[q][i]), floor_at);
@@ -415,10 +460,14 @@ Split choose_split(const Geometry& g, int F, int C, const int (&at_once)[4]) {
     // 128 x 32 take 49 and 41, 256 x 64 by a pair 45)
     const double step = std::max(BN / 2.0, cg == 2 ? 36.0 + BN / 8.0 : 36.0 + BN / 4.0);
     const double fill = 3000.0, tail = (4 * BN > 512 || rounds == 1) ? 8.0 * BN : 0.0;
-    const double t = fill + rounds * (steps * step / parts + tail) + (parts > 1 ? 2500.0 + 4.0 * BN : 0.0);
+    // sums of several chunks: adding one up holds the tensor core up unless there is a second accumulator set
+    const int chunks = (ncb / parts + CHUNK - 1) / CHUNK;
+    const double adding = chunks > 1 && 6 * BN > 512 ? 16.0 * BN * (chunks - 1) : 0.0;
+    const double t = fill + rounds * (steps * step / parts + tail + adding) + (parts > 1 ? 2500.0 + 4.0 * BN : 0.0);
     if (t < best_t) { best_t = t; best = Split{cg, BN, groups, parts}; }
   };
-  for (int groups = (F + 255) / 256; groups <= (F + 31) / 32; groups *= 2) consider(2, groups, 1);
+  const int most = ncb > CHUNK ? 128 : 256;
+  for (int groups = (F + most - 1) / most; groups <= (F + 31) / 32; groups *= 2) consider(2, groups, 1);
   for (int groups = (F + 127) / 128; groups <= (F + 15) / 16; groups *= 2)
     for (int parts = 1; parts <= MAX_PARTS_MMA && parts <= ncb; parts *= 2) consider(1, groups, parts);
   return best;
@@ -445,7 +494,7 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   if (!dv) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cannot query the current device");
   Params p;
   using KernelFn = void (*)(const Maps, const Params);
-  static const KernelFn kernels[2] = {k_conv_mma_f16<1>, k_conv_mma_f16<2>};
+  static const KernelFn kernels[4] = {k_conv_mma_f16<1, false>, k_conv_mma_f16<2, false>, k_conv_mma_f16<1, true>, k_conv_mma_f16<2, true>};
   static thread_local int at_once[kMaxDevices][4];
   const int di = (int)(dv - slots);
   if (!dv->ready) {
@@ -513,7 +562,7 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 2;
   cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = SMEM_BYTES;
   cfg.gridDim = dim3((unsigned)(sp.parts > 1 ? p.items * sp.parts : sp.cg * std::min(p.items, at_once[di][sp.cg - 1])));
-  if (int rc = check_cuda(cudaLaunchKernelEx(&cfg, kernels[sp.cg - 1], maps, p), "pat_conv3x3 launch")) return rc;
+  if (int rc = check_cuda(cudaLaunchKernelEx(&cfg, kernels[sp.cg - 1 + (p.ncb > CHUNK ? 2 : 0)], maps, p), "pat_conv3x3 launch")) return rc;
   count_launches(1);
   return check_cuda(cudaGetLastError(), "pat_conv3x3 launch");
 }

@@ -235,3 +235,30 @@ def test_an_infinite_input_reaches_only_the_kept_taps(case, dtype):
     assert pc.pat_query_status() == 0
     x.fill_(float("nan"))                      # every output is formed again
     assert torch.equal(torch.isnan(call()), conv(torch.ones_like(x), wd != 0) > 0.5) and pc.pat_query_status() == 0
+
+
+# CTA pairs over whole sums, one round and several; channels cut among the CTAs of a cluster; a short last chunk
+@pytest.mark.parametrize("case", [(64, 28, 28, 4608, 64), (16, 28, 28, 1096, 256), (64, 14, 14, 2560, 320), (1, 14, 14, 8192, 64)], ids=lambda c: "-".join(str(v) for v in c))
+def test_f16_long_sums_do_not_drift(case):
+    """Positive data: a sum that only ever drops bits ends low by a share that grows with its length."""
+    N, H, W, C, F = case
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(C)
+    w = torch.rand((F, C, 3, 3), generator=gen, device="cuda") / C
+    x = torch.rand((N, H, W, C), generator=gen, device="cuda").to(torch.float16)
+    masks = pc.pat_library_builtin(4)
+    pid, wm = pc.pat_project(w, masks, F * C)
+    blob = pc.pat_pack(wm, pid, masks, F * C, "f16")
+    y = pc.pat_conv3x3(blob, F, C, masks, F * C, "f16", x, 1)
+    assert pc.pat_query_status() == 0
+    wd = pc.pat_unpack(blob, F, C, masks, F * C, "f16").double()
+    low, total, n = 0.0, 0.0, 0
+    for i in sorted({0, N // 2, N - 1}):
+        ref = Fn.conv2d(x[i:i + 1].permute(0, 3, 1, 2).double(), wd, padding=1).permute(0, 2, 3, 1)
+        err = y[i:i + 1].double() - ref
+        # 512 channels are 288 steps; a step drops less than two units in the last place of its running sum
+        assert bool((err.abs() <= (F16_ROUND + 288 * 2 * STEP) * ref).all())
+        low, total, n = low + float(err.sum()), total + float(ref.sum()), n + ref.numel()
+    # in the mean one of the two, of a running sum that is half of the whole in the mean; roundings of the results (at most
+    # 2^-11, either way) leave five of their standard deviations
+    assert abs(low) <= (288 * STEP / 2 + 5 * F16_ROUND / (3 * n) ** 0.5) * total
