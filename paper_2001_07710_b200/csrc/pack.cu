@@ -208,6 +208,7 @@ template <> __device__ inline void dense_store<float>(uint32_t* dst, size_t term
 // in flight: without the bound 178 registers, 43 instead of 28 us a call.  The work before the wait took the call from 10.3 to
 // 8.0 us at 64 x 64, 16.9 to 14.0 at 512 x 512 (fp16).
 constexpr int kScatterThreads = 256, kListThreads = 128;
+constexpr size_t kScatterStatic = 1024;    // static shared memory
 template <typename T, bool TABLE>
 __global__ void __launch_bounds__(kScatterThreads, 5) k_pack_scatter(const float* __restrict__ wm, const uint8_t* __restrict__ pid,
                                                                   int C, int K, int nct, bool blocks, MaskTable lib, BlobPtrs bp) {
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(kScatterThreads, 5) k_pack_scatter(const float
   const int words = (nct + 31) / 32;
   uint8_t* spid = reinterpret_cast<uint8_t*>(stage_bits + (blocks ? 2 * words : 0));        // C pattern ids of this filter
   __shared__ int s_pptr[kMaxK];
+  static_assert(sizeof(s_pptr) <= kScatterStatic, "what pat_pack counts with");
   const int f = blockIdx.x, tid = threadIdx.x;
   for (int c = tid; c < C; c += kScatterThreads) spid[c] = pid[(size_t)f * C + c];
   if (TABLE)
@@ -548,19 +550,19 @@ extern "C" int pat_pack(const float* w_masked, const uint8_t* pattern_id, int F,
   // every check that can refuse the call comes before the first launch
   const size_t table = sizeof(int) * (size_t)L.nct * K;
   const bool use_table = table <= 24 * 1024;
-  const size_t smem = (use_table ? table : 0) + sizeof(int) * ((size_t)L.nct + 1 + (L.nblk ? 2 * (((size_t)L.nct + 31) / 32) : 0)) + (size_t)C;
-  if (smem > 48 * 1024) return set_error(PAT_ERR_SHAPE, "pat_pack: C=%d too large for the packing kernel", C);
+  const size_t lists = (use_table ? table : 0) + sizeof(int) * ((size_t)L.nct + 1) + (size_t)C;
+  if (lists > 48 * 1024) return set_error(PAT_ERR_SHAPE, "pat_pack: C=%d too large for the packing kernel", C);
+  const size_t smem = lists + sizeof(int) * (L.nblk ? 2 * (((size_t)L.nct + 31) / 32) : 0);
+  const auto scatter = dtype == PAT_F16 ? (use_table ? k_pack_scatter<__half, true> : k_pack_scatter<__half, false>)
+                                        : (use_table ? k_pack_scatter<float, true> : k_pack_scatter<float, false>);
+  // with the kernel's static arrays the last of these sizes are above what a launch gets without asking
+  if (smem + kScatterStatic > 48 * 1024)
+    if (int rc = check_cuda(cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "set shared memory size")) return rc;
   cudaError_t le = cudaSuccess;                   // first launch error, if any
   auto note = [&](cudaError_t e) { if (le == cudaSuccess) le = e; };
   note(launch_dependent(k_pack_count, dim3(F), dim3(256), K * sizeof(int), st, pattern_id, C, K, bp, status));
   note(launch_dependent(k_pack_rank, dim3(F), dim3(kRankThreads), 0, st, F, C, K, (long long)n_keep, dtype, lib, (unsigned long long)L.total, bp, status));
-  if (dtype == PAT_F16) {
-    if (use_table) note(launch_dependent(k_pack_scatter<__half, true>, dim3(F), dim3(256), smem, st, w_masked, pattern_id, C, K, L.nct, L.nblk > 0, lib, bp));
-    else note(launch_dependent(k_pack_scatter<__half, false>, dim3(F), dim3(256), smem, st, w_masked, pattern_id, C, K, L.nct, L.nblk > 0, lib, bp));
-  } else {
-    if (use_table) note(launch_dependent(k_pack_scatter<float, true>, dim3(F), dim3(256), smem, st, w_masked, pattern_id, C, K, L.nct, L.nblk > 0, lib, bp));
-    else note(launch_dependent(k_pack_scatter<float, false>, dim3(F), dim3(256), smem, st, w_masked, pattern_id, C, K, L.nct, L.nblk > 0, lib, bp));
-  }
+  note(launch_dependent(scatter, dim3(F), dim3(kScatterThreads), smem, st, w_masked, pattern_id, C, K, L.nct, L.nblk > 0, lib, bp));
   count_launches(3);
   if (L.nblk > 0) {
     note(launch_dependent(k_pack_blocks, dim3(L.nblk), dim3(32), 0, st, L.nct, L.nblk, lib, bp));
