@@ -122,6 +122,19 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
   cfg.attrs = &attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+// The launches of a call, one after the other: behind one that failed nothing is launched (what it should have written would
+// be read, as offsets too).
+struct Launches {
+  cudaError_t error = cudaSuccess;
+  int n = 0;
+  template <typename... Args>
+  void add(Args&&... args) { add_result([&] { return launch_dependent(static_cast<Args&&>(args)...); }); }
+  template <typename Launch>
+  void add_result(Launch&& launch) {
+    if (error == cudaSuccess) error = launch();
+    if (error == cudaSuccess) ++n;
+  }
+};
 #ifdef __CUDACC__
 // After the wait the kernel's own dependents may be launched: they wait here in turn (for the whole of this kernel), and
 // everything before it has completed.

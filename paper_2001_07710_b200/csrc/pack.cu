@@ -558,17 +558,13 @@ extern "C" int pat_pack(const float* w_masked, const uint8_t* pattern_id, int F,
   // with the kernel's static arrays the last of these sizes are above what a launch gets without asking
   if (smem + kScatterStatic > 48 * 1024)
     if (int rc = check_cuda(cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "set shared memory size")) return rc;
-  cudaError_t le = cudaSuccess;                   // first launch error, if any
-  auto note = [&](cudaError_t e) { if (le == cudaSuccess) le = e; };
-  note(launch_dependent(k_pack_count, dim3(F), dim3(256), K * sizeof(int), st, pattern_id, C, K, bp, status));
-  note(launch_dependent(k_pack_rank, dim3(F), dim3(kRankThreads), 0, st, F, C, K, (long long)n_keep, dtype, lib, (unsigned long long)L.total, bp, status));
-  note(launch_dependent(scatter, dim3(F), dim3(kScatterThreads), smem, st, w_masked, pattern_id, C, K, L.nct, L.nblk > 0, lib, bp));
-  count_launches(3);
-  if (L.nblk > 0) {
-    note(launch_dependent(k_pack_blocks, dim3(L.nblk), dim3(32), 0, st, L.nct, L.nblk, lib, bp));
-    count_launches(1);
-  }
-  if (le != cudaSuccess) return check_cuda(le, "pat_pack launch");
+  Launches launches;
+  launches.add(k_pack_count, dim3(F), dim3(256), K * sizeof(int), st, pattern_id, C, K, bp, status);
+  launches.add(k_pack_rank, dim3(F), dim3(kRankThreads), 0, st, F, C, K, (long long)n_keep, dtype, lib, (unsigned long long)L.total, bp, status);
+  launches.add(scatter, dim3(F), dim3(kScatterThreads), smem, st, w_masked, pattern_id, C, K, L.nct, L.nblk > 0, lib, bp);
+  if (L.nblk > 0) launches.add(k_pack_blocks, dim3(L.nblk), dim3(32), 0, st, L.nct, L.nblk, lib, bp);
+  count_launches(launches.n);
+  if (launches.error != cudaSuccess) return check_cuda(launches.error, "pat_pack launch");
   return check_cuda(cudaGetLastError(), "pat_pack launch");
 }
 

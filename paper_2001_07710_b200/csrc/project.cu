@@ -624,14 +624,13 @@ extern "C" int pat_project(const float* w, int F, int C, const uint16_t* masks, 
   int mode = -1;
   if (n_keep == FC) mode = 1;
   else if (n_keep == 0) mode = 0;
-  cudaError_t le = cudaSuccess;                   // first launch error, if any
-  auto note = [&](cudaError_t e) { if (le == cudaSuccess) le = e; };
+  Launches launches;
   static_assert(kHistWords % 4 == 0 && (kBins + kCoarse) % 4 == 0, "counters are zeroed four at a time");
-  if (mode < 0) note(launch_dependent(k_zero_counters, dim3((unsigned)((kHistWords / 4 + kZeroThreads - 1) / kZeroThreads)), dim3(kZeroThreads), 0, st, ws.hist, (int)kHistWords));
-  note(launch_dependent(k_select_pattern, dim3(nb_sel), dim3(kPatBlock), 0, st, w, FC, lib, ws.key, ws.pid, ws.hist, mode < 0));
+  if (mode < 0) launches.add(k_zero_counters, dim3((unsigned)((kHistWords / 4 + kZeroThreads - 1) / kZeroThreads)), dim3(kZeroThreads), 0, st, ws.hist, (int)kHistWords);
+  launches.add(k_select_pattern, dim3(nb_sel), dim3(kPatBlock), 0, st, w, FC, lib, ws.key, ws.pid, ws.hist, mode < 0);
   if (mode < 0) {
     if (FC <= kBlockKeys) {
-      note(launch_dependent(k_select_cluster<1>, dim3(1), dim3(kSelThreads), 0, st, ws.key, FC, ws.st, (long long)n_keep, ws.hist));
+      launches.add(k_select_cluster<1>, dim3(1), dim3(kSelThreads), 0, st, ws.key, FC, ws.st, (long long)n_keep, ws.hist);
     } else if (FC <= kClusterKeys) {
       cudaLaunchAttribute attr[2];
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -640,15 +639,17 @@ extern "C" int pat_project(const float* w, int F, int C, const uint16_t* masks, 
       attr[1].val.clusterDim.x = kSelBlocks; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(kSelBlocks); cfg.blockDim = dim3(kSelThreads); cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 2;
-      note(cudaLaunchKernelEx(&cfg, k_select_cluster<kSelBlocks>, static_cast<const unsigned long long*>(ws.key), FC, ws.st, (long long)n_keep,
-                              static_cast<const unsigned int*>(ws.hist)));
+      launches.add_result([&] {
+        return cudaLaunchKernelEx(&cfg, k_select_cluster<kSelBlocks>, static_cast<const unsigned long long*>(ws.key), FC, ws.st, (long long)n_keep,
+                                  static_cast<const unsigned int*>(ws.hist));
+      });
     } else {
-      note(launch_dependent(k_select_rest, dim3(nb_rest), dim3(kRestThreads), 0, st, ws.key, FC, ws.st, (long long)n_keep, ws.hist, ws.cand_key, ws.cand));
+      launches.add(k_select_rest, dim3(nb_rest), dim3(kRestThreads), 0, st, ws.key, FC, ws.st, (long long)n_keep, ws.hist, ws.cand_key, ws.cand);
     }
   }
-  note(launch_dependent(k_finalize, dim3(nblk), dim3(kSelBlock), 0, st, w, FC, lib, ws.key, ws.pid, ws.st, pattern_id, w_masked, mode));
-  count_launches(mode < 0 ? 4 : 2);
-  if (le != cudaSuccess) return check_cuda(le, "pat_project launch");
+  launches.add(k_finalize, dim3(nblk), dim3(kSelBlock), 0, st, w, FC, lib, ws.key, ws.pid, ws.st, pattern_id, w_masked, mode);
+  count_launches(launches.n);
+  if (launches.error != cudaSuccess) return check_cuda(launches.error, "pat_project launch");
   return check_cuda(cudaGetLastError(), "pat_project launch");
 }
 
