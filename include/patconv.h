@@ -265,10 +265,10 @@ int pat_argmax_binarize(const float *z, int64_t n, int K, uint8_t *index_out, fl
 int pat_extract_library(const float *w, int64_t n, const uint16_t *masks_in, int K_in, int K_out,
                         uint16_t *masks_out, uint64_t *counts_out, void *stream);
 
-/* Test hooks of the convolution kernels' bounded waits (host-side, process-wide, not thread safe).  The paper has
- * no counterpart.
+/* Test hooks of the tensor-core convolutions' bounded waits (host-side, process-wide, not thread safe).  The paper has
+ * no counterpart.  (The fp32 multiply-add kernel has neither: its limit is the default.)
  *   what = 0  limit of every device-side wait in nanoseconds (value <= 0: back to the default of 2 s);
- *   what = 1  tensor-core and workspace kernels: in every thread block the copy of pipeline stage number `value`
+ *   what = 1  in every thread block the copy of pipeline stage number `value`
  *             is never issued, so the wait for it runs out after the limit and the kernel ends, with every other
  *             copy landed and its tensor memory released, leaving PAT_ERR_TIMEOUT in the status word
  *             (value < 0: off, the default).

@@ -179,6 +179,25 @@ def test_a_result_that_is_not_a_number_stays_one(case, dtype):
     assert pc.pat_query_status() == 0
 
 
+@pytest.mark.parametrize("C,channel", [(32, 5), (32, 20), (64, 40), (72, 70)])
+def test_f32_one_product_per_output(C, channel):
+    """One non-zero channel in either half of a block of 32 and in a short last one: each output is at most four products, so
+    that every one of the six products of parts shows."""
+    F, H = 48, 12
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(C + channel)
+    w = torch.randn((F, C, 3, 3), generator=gen, device="cuda")
+    masks = pc.pat_library_builtin(4)
+    pid, wm = pc.pat_project(w, masks, F * C)
+    blob = pc.pat_pack(wm, pid, masks, F * C, "f32")
+    x = torch.zeros((2, H, H, C), device="cuda")
+    x[:, ::3, ::3, channel] = torch.randn((2, H // 3, H // 3), generator=gen, device="cuda")       # three apart: one product each
+    y = pc.pat_conv3x3(blob, F, C, masks, F * C, "f32", x, 1)
+    ref = Fn.conv2d(x.permute(0, 3, 1, 2).double(), wm.double(), padding=1).permute(0, 2, 3, 1)
+    # three products of parts left out, below 2^-25 together; six added up with at most a unit in the last place each
+    assert bool(((y.double() - ref).abs() <= 6 * STEP * ref.abs()).all())
+
+
 @pytest.mark.parametrize("value", [3.4028234e38, -3.4e38, 3.3961e38])
 def test_f32_largest_weights(value):
     """Weights that bf16 would round to infinity."""
@@ -262,3 +281,31 @@ def test_f16_long_sums_do_not_drift(case):
     # in the mean one of the two, of a running sum that is half of the whole in the mean; roundings of the results (at most
     # 2^-11, either way) leave five of their standard deviations
     assert abs(low) <= (288 * STEP / 2 + 5 * F16_ROUND / (3 * n) ** 0.5) * total
+
+
+# every way in which the kernels are run: weights resident, CTA pairs over a ring, channels cut among a cluster's CTAs, sums over
+# several chunks; fp32 pairs and clusters; with pooling, whose epilogue warps meet at barriers
+@pytest.mark.parametrize("dtype,case", [("f16", (4, 56, 56, 64, 64, 8, 0.125, 1, 0)), ("f16", (24, 28, 28, 256, 512, 8, 0.125, 1, 1)),
+                                        ("f16", (1, 14, 14, 512, 512, 8, 0.125, 1, 2)), ("f16", (16, 28, 28, 1096, 256, 8, 0.125, 1, 0)),
+                                        ("f32", (24, 28, 28, 256, 256, 8, 0.25, 1, 2)), ("f32", (1, 14, 14, 512, 512, 8, 0.25, 1, 0)),
+                                        ("f32", (4, 29, 29, 64, 64, 8, 0.25, 2, 1))], ids=str)
+def test_a_wait_that_runs_out_ends_the_kernel(dtype, case):
+    """The weights of one stage are never copied (test hook) and the waits are limited to 1 ms: the call ends by itself with a
+    status, and the next one is correct."""
+    N, H, W, C, F, K, keep, stride, act = case
+    masks, n_keep = pc.pat_library_builtin(K), int(F * C * keep)
+    pid, wm = pc.pat_project(torch.ones((F, C, 3, 3), device="cuda"), masks, n_keep)
+    blob = pc.pat_pack(wm, pid, masks, n_keep, dtype)
+    x = torch.ones((N, H, W, C), dtype=torch.float16 if dtype == "f16" else torch.float32, device="cuda")
+    try:
+        pc.pat_debug_set(0, 1_000_000)
+        pc.pat_debug_set(1, 1)
+        pc.pat_conv3x3(blob, F, C, masks, n_keep, dtype, x, stride, relu=act == 1, pool=act == 2)
+        with pytest.raises(pc.PatError) as e:
+            pc.pat_query_status()
+        assert e.value.code == 9
+    finally:
+        pc.pat_debug_set(1, -1)
+        pc.pat_debug_set(0, 0)
+    assert pc.pat_query_status() == 0
+    check(case, dtype)
