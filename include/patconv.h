@@ -144,9 +144,10 @@ int pat_unpack(const void *blob, int F, int C, const uint16_t *masks, int K, int
  *   Y[n][y][x][f] = sum over kept kernels (f,c) and their four taps (r,s) of
  *                   w[f][c][r][s] * X[n][y*stride + r - 1][x*stride + s - 1][c]
  * Sums are fp32 and so are the products: fp16 inputs are multiplied exactly, fp32 inputs as three bf16 parts each, of whose
- * products those below 2^-25 of the result's terms are left out.  The tensor cores' own sums drop what does not fit their last
- * bit; they run over 512 channels in fp16 and 32 in fp32 at most and are added up rounded to nearest.  The result is stored in the blob's dtype (fp16: round to
- * nearest even).
+ * products those below 2^-25 of the result's terms are left out (parts below 2^-133 are lost: values below 2^-117 count to
+ * within 2^-134).  The tensor cores' own sums drop what does not fit their last bit; they run over 512 channels in fp16 and
+ * 32 in fp32 at most and are added up rounded to nearest.  The result is stored in the blob's dtype (fp16: round to nearest
+ * even).
  * F and C multiples of eight: the tensor cores run the dense form of the masked weights, zeros included.  An infinity or NaN
  * reaches the outputs whose kept taps read it and no others all the same: results that the zeros would make NaN are formed
  * again from the kept taps, which takes its time when there are many.
@@ -164,7 +165,7 @@ int pat_conv3x3(const void *blob, int F, int C, const uint16_t *masks, int K, in
  * the bytes that the shape may need (about 1.3 x the size of x, plus 59 MB for partial sums; for C a multiple of 16, F a
  * multiple of 32, W a multiple of 14 with W/14 in {1, 2, 4k} or W < 14, max(ceil(H/4), 4) == 4 or >= 7, either dtype and
  * stride), or 0 for a shape that never uses one: pat_conv3x3_ws then behaves exactly like pat_conv3x3 and ignores the
- * workspace.
+ * workspace.  A call needs that workspace whichever kernels run it; fp16 and stride 2 read none of it.
  *   workspace  dev, at least pat_conv3x3_workspace(...) bytes, 256-byte aligned; contents are scratch;
  *              concurrent calls must use different workspaces
  * Results: those of pat_conv3x3, added in fp32 in an order that may differ. */
@@ -180,8 +181,8 @@ int pat_conv3x3_ws(const void *blob, int F, int C, const uint16_t *masks, int K,
  * act = 2 fuses the 2 x 2 max pooling that follows five of the thirteen layers of the VGG-16 of Section 7 as well:
  * y is then NHWC [N][H/2][W/2][F] and holds max(0, the four results of each 2 x 2 block) - the values of
  * pat_relu_maxpool(pool = 1) on the output of act = 0, bit for bit (rounding is monotone) - and the full-size
- * output is never written.  act = 2 needs stride 1, even H and W and a shape with a workspace
- * (pat_conv3x3_workspace(...) > 0): PAT_ERR_SHAPE otherwise, nothing launched; such a layer takes act = 1 and a
+ * output is never written.  A NaN becomes zero with either, as in pat_relu_maxpool.  act = 2 needs stride 1, even H and W
+ * and a shape with a workspace (pat_conv3x3_workspace(...) > 0): PAT_ERR_SHAPE otherwise, nothing launched; such a layer takes act = 1 and a
  * separate pat_relu_maxpool.  Other arguments, errors and workspace as for pat_conv3x3_ws; PAT_ERR_INVALID_ARG for
  * any other `act`. */
 int pat_conv3x3_ws_act(const void *blob, int F, int C, const uint16_t *masks, int K, int64_t n_keep,
@@ -211,8 +212,9 @@ int pat_query_status(void *stream);
  * all entry points).  Host-side counter; useful to check that work really ran on the GPU. */
 uint64_t pat_launch_count(void);
 
-/* Measures the device's multiply-add rate (kind 0: fma.rn.f32, kind 1: fma.rn.f32.f16 with an fp32 accumulator): the
- * denominator of the multiply-add kernels' roofline, taken at the clock the device really runs at.  Launches a few short kernels on `stream` and waits for them (this one call synchronises).
+/* Measures the device's multiply-add rate (kind 0: fma.rn.f32, what the fp32 multiply-add kernels issue; kind 1:
+ * fma.rn.f32.f16 with an fp32 accumulator, which no kernel of the library issues): the denominator of those kernels' roofline,
+ * taken at the clock the device really runs at.  Launches a few short kernels on `stream` and waits for them (this one call synchronises).
  *   scratch     dev, 256-byte aligned, at least 256 + 4 * 8 * 256 * (number of SMs) bytes (2 MiB always suffices)
  *   tflops_out  host out: best of three runs, in TFLOP/s (2 flop per multiply-add)
  * The paper has no counterpart (it reports end-to-end latencies, Section 7.2). */

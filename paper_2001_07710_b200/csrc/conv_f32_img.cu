@@ -135,7 +135,7 @@ __device__ __forceinline__ void lds_row_f32(float (&h)[16], uint32_t a, uint32_t
   }
 }
 
-// The code of one pattern on a 4 x 14 tile (see pattern_body4 in conv_tile.cuh): a0 = address of logical chunk 0 of
+// The code of one pattern on a 4 x 14 tile: a0 = address of logical chunk 0 of
 // window row `sh`, swb = the lane's chunk swizzle (bits 4-5) for window rows 0-3; from window row 4 on the rows
 // belong to the next tile row's group, whose parity bit is the other one.
 template <uint32_t MASK>
@@ -357,7 +357,7 @@ __device__ __forceinline__ void conv_body(const Params& p, unsigned char* smem) 
 #pragma unroll 1
       for (;;) {
         // all lanes hold the same descriptor word; the warp-wide reduction makes that known to the compiler, so that
-        // the branches of this visit are uniform branches without reconvergence bookkeeping 
+        // the branches of this visit are uniform branches without reconvergence bookkeeping
         const uint32_t cm = __reduce_or_sync(0xFFFFFFFFu, m0), coff = off;
         float w[4] = {__uint_as_float(w0), __uint_as_float(w1), __uint_as_float(w2), __uint_as_float(w3)};
         float r0[16];                      // the first window row of this kernel (window rows 0-3 share the lane's swizzle)
