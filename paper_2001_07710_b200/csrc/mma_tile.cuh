@@ -271,10 +271,11 @@ struct Note {                              // zero as long as all values seen we
     } else {
       const __half2 z = __float2half2_rn(0.0f);
       const __half2* h = reinterpret_cast<const __half2*>(&v);
-      __half2 s = *reinterpret_cast<__half2*>(&t.x);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) s = __hfma2(h[i], z, s);
-      t.x = *reinterpret_cast<float*>(&s);
+      __half2 s0 = *reinterpret_cast<__half2*>(&t.x), s1 = *reinterpret_cast<__half2*>(&t.y);     // (two chains)
+      s0 = __hfma2(h[2], z, __hfma2(h[0], z, s0));
+      s1 = __hfma2(h[3], z, __hfma2(h[1], z, s1));
+      t.x = *reinterpret_cast<float*>(&s0);
+      t.y = *reinterpret_cast<float*>(&s1);
     }
   }
   // (floats or pairs of halves, each of either sign's zero or NaN)
