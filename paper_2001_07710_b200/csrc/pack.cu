@@ -555,9 +555,11 @@ extern "C" int pat_pack(const float* w_masked, const uint8_t* pattern_id, int F,
   const size_t smem = lists + sizeof(int) * (L.nblk ? 2 * (((size_t)L.nct + 31) / 32) : 0);
   const auto scatter = dtype == PAT_F16 ? (use_table ? k_pack_scatter<__half, true> : k_pack_scatter<__half, false>)
                                         : (use_table ? k_pack_scatter<float, true> : k_pack_scatter<float, false>);
-  // with the kernel's static arrays the last of these sizes are above what a launch gets without asking
+  // with the kernel's static arrays the last of these sizes are above what a launch gets without asking (always the same value:
+  // another thread may be packing another size)
+  constexpr int kScatterMost = 49 * 1024;    // lists of 48 KB leave room for 616 bytes of stage bits at most
   if (smem + kScatterStatic > 48 * 1024)
-    if (int rc = check_cuda(cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "set shared memory size")) return rc;
+    if (int rc = check_cuda(cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, kScatterMost), "set shared memory size")) return rc;
   Launches launches;
   launches.add(k_pack_count, dim3(F), dim3(256), K * sizeof(int), st, pattern_id, C, K, bp, status);
   launches.add(k_pack_rank, dim3(F), dim3(kRankThreads), 0, st, F, C, K, (long long)n_keep, dtype, lib, (unsigned long long)L.total, bp, status);
