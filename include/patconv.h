@@ -121,8 +121,8 @@ size_t pat_pack_size(int F, int C, int K, int64_t n_keep, int dtype);
  *   w4[n_keep][4]      the four kept entries in ascending bit order, fp32, or fp16 rounded to
  *                      nearest-even when dtype = PAT_F16
  * followed by sections that only the convolution reads: the kernels re-sorted by blocks of 16 input channels, and for
- * layers whose F and C are multiples of eight the masked weights in dense form, laid out for the tensor cores (fp16, or
- * fp32 as three bf16 numbers).
+ * layers with F a multiple of eight and C one of four the masked weights in dense form, laid out for the tensor cores (fp16,
+ * or fp32 as three bf16 numbers).
  *   w_masked, pattern_id  dev, as written by pat_project; exactly n_keep kernels must be kept
  *   blob        dev out, at least pat_pack_size(...) bytes, 256-byte aligned */
 int pat_pack(const float *w_masked, const uint8_t *pattern_id, int F, int C,
@@ -148,7 +148,7 @@ int pat_unpack(const void *blob, int F, int C, const uint16_t *masks, int K, int
  * within 2^-134).  The tensor cores' own sums drop what does not fit their last bit; they run over 512 channels in fp16 and
  * 32 in fp32 at most and are added up rounded to nearest.  The result is stored in the blob's dtype (fp16: round to nearest
  * even).
- * F and C multiples of eight: the tensor cores run the dense form of the masked weights, zeros included.  An infinity or NaN
+ * F a multiple of eight, C one of four: the tensor cores run the dense form of the masked weights, zeros included.  An infinity or NaN
  * reaches the outputs whose kept taps read it and no others all the same: results that the zeros would make NaN are formed
  * again from the kept taps, which takes its time when there are many.
  *   blob     dev, written by pat_pack with the same (F, C, masks, K, n_keep, dtype)

@@ -44,7 +44,7 @@ struct BlobLayout {
   size_t xfilt, tptr, tmeta, tw4;      // execution section (its own filter order, see pack.cu)
   size_t dboff, dblk;                  // descriptor blocks (img_blocks; else empty)
   int nblk;                            // number of descriptor blocks = (F / 32) * (C / 8), or 0
-  size_t dense;                        // masked weights in dense form for the tensor cores (see mma_weights)
+  size_t dense;                        // masked weights in dense form for the tensor cores (see mma_weights); 0: none
   size_t scratch;                      // pack-time temporaries: hist[F][K], count[F], inv[F] (kept, see inv_offset), xinv[F], xbase[F], stage bits
   size_t total;
   int nct;                             // number of 16-channel tiles = ceil(C / 16)
@@ -53,13 +53,15 @@ struct BlobLayout {
 __host__ __device__ inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 __host__ __device__ inline int elem_bytes(int dtype) { return dtype == PAT_F16 ? 2 : 4; }
 
-// Layers that the tensor cores run (16-byte rows of activations, weights and results); their blobs hold the masked weights in
-// dense form as well: [terms][9][F][pitch of C] 16-bit values, fp16 as they are stored (one term), fp32 as the sum of
-// three bf16 numbers (8 bits of the 24 each).
+// Layers that the tensor cores run (results in pieces of 16 bytes, activations in pieces of four channels); their blobs hold
+// the masked weights in dense form as well: [terms][9][F][pitch of C] 16-bit values, fp16 as they are stored (one term), fp32 as
+// the sum of three bf16 numbers (8 bits of the 24 each).  With C an odd multiple of four the dense form stands at the end of the
+// blob: blobs of such layers that were packed when they had none hold the same at the same places, but for it
+// (dense_form_end).
 constexpr int kMmaTermsF32 = 3;
 __host__ __device__ inline int mma_terms(int dtype) { return dtype == PAT_F16 ? 1 : kMmaTermsF32; }
 __host__ __device__ inline int mma_pitch(int C) { return (C + 7) / 8 * 8; }
-__host__ __device__ inline bool mma_weights(int F, int C) { return F % 8 == 0 && C % 8 == 0; }
+__host__ __device__ inline bool mma_weights(int F, int C) { return F % 8 == 0 && C % 4 == 0; }
 // Layers whose blobs hold descriptor blocks for the multiply-add workspace kernels: fp32 at low density.  Which of the two
 // runs is decided per call by the sizes (conv_api.cu); above one kernel in six the tensor cores won at every size
 // (56x56x256 -> 256, batch 32, keep 3/16: 346 against 379 us), and in fp16 at every density down to 1 %
@@ -88,11 +90,17 @@ __host__ __device__ inline BlobLayout blob_layout(int F, int C, int K, int64_t n
   L.nblk = has_blocks ? (F / kExecGroup) * (C / kChanStageF32) : 0;
   L.dboff = o; o = align256(o + (L.nblk ? sizeof(uint32_t) * ((size_t)L.nblk + 1) : 0));
   L.dblk = o;  o = align256(o + (L.nblk ? (size_t)L.nblk * (kBlockHeaderBytes + op_bytes * kBlockWarps) + op_bytes * nk : 0));
-  L.dense = o;  o = align256(o + (mma_weights(F, C) ? 9 * 2 * (size_t)mma_terms(dtype) * F * mma_pitch(C) : 0));
+  const size_t dense_bytes = mma_weights(F, C) ? 9 * 2 * (size_t)mma_terms(dtype) * F * mma_pitch(C) : 0;
+  L.dense = dense_bytes ? o : 0;
+  if (C % 8 == 0) o = align256(o + dense_bytes);
   L.scratch = o; o = align256(o + sizeof(int32_t) * (size_t)F * ((size_t)K + 4 + (L.nblk ? 2 * (((size_t)L.nct + 31) / 32) : 0)));
+  if (dense_bytes && C % 8 != 0) { L.dense = o; o = align256(o + dense_bytes); }
   L.total = o;
   return L;
 }
+
+// A blob of a layer with C an odd multiple of four is this long when it holds the dense form (0: other layers).
+__host__ __device__ inline uint64_t dense_form_end(const BlobLayout& L, int C) { return L.dense && C % 8 != 0 ? L.total : 0; }
 
 // inv[F]: original filter -> its position in the canonical order.
 __host__ __device__ inline size_t inv_offset(const BlobLayout& L, int F, int K) { return L.scratch + sizeof(int32_t) * (size_t)F * ((size_t)K + 1); }

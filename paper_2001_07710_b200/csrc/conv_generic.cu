@@ -1,7 +1,7 @@
 // Generic sparse / dense 3x3 convolution kernels: any shape, stride 1 or 2, fp32 or fp16 storage.
 //
-// These are the shape-agnostic kernels of the library: sparse layers whose channels or filters are not multiples of eight
-// (the others run on the tensor cores, conv_mma_f16.cu and conv_mma_f32.cu), and the dense first layer.  Mapping of the sparse kernel:
+// These are the shape-agnostic kernels of the library: sparse layers whose filters are not a multiple of eight or channels not one
+// of four (the others run on the tensor cores, conv_mma_f16.cu and conv_mma_f32.cu), and the dense first layer.  Mapping of the sparse kernel:
 // a thread block owns an 8 x 32
 // tile of output pixels and 32 re-ordered filters; lanes run along x so every weight is warp-uniform; each
 // thread keeps an 8-row column of outputs for 4 filters in registers.  Activations are staged 16 input

@@ -25,6 +25,11 @@
 // data: 1.2e-5 low, against 2^-11 of rounding the result); further chunks are added up, rounded to nearest, in columns of
 // tensor memory of their own, which halves the filters that a pair takes.
 //
+// Channels an odd multiple of four (ROWS8): activation rows start at multiples of 8 bytes only, which TMA does not take; four
+// warps then fill the same buffers with 8-byte cp.async (four: eight are no faster, the epilogue spills; 56x56x68 -> 200, batch 16:
+// 41 us, 72 channels through TMA 25: the copies' issue bounds it).  These layers ran the generic multiply-add kernel before:
+// 28x28x260 -> 256, batch 32 508 -> 47 us, 9x10x212 -> 152, batch 8 255 -> 13, 80x81x20 -> 24, stride 2, batch 2 64 -> 16.
+//
 // Roles: warps 0-7 epilogue (tensor memory -> fp32 -> rectifier -> fp16 -> shared memory -> coalesced stores), warp 8
 // copies activations, warp 9 weights, warp 10 issues the multiply-adds (in the even CTA of a pair).  Every wait is
 // bounded; tensor memory is released on every path.
@@ -36,7 +41,9 @@ namespace {
 
 constexpr int TILE = 256;                   // positions per CTA
 constexpr int KB = 64;                      // channels per stage (128 bytes)
-constexpr int W_A = 8, W_B = 9, W_MMA = 10, NWARPS = 12, NTHREADS = NWARPS * 32;
+constexpr int W_A = 8, W_B = 9, W_MMA = 10, NWARPS = 12;
+constexpr int ROW_WARPS = 4;                // ROWS8: warps that copy activations (W_A and those behind W_MMA)
+constexpr int threads_of(bool rows8) { return (rows8 ? W_MMA + ROW_WARPS : NWARPS) * 32; }
 constexpr int MAX_A = 4, MAX_B = 8;             // ring slots
 constexpr int CHUNK = 8;                        // channel blocks in one sum of the tensor core
 constexpr int ST_BYTES = TILE * 128;            // epilogue staging: 128 bytes per position
@@ -53,8 +60,8 @@ struct Params : Geometry {
 };
 
 // LONG: more than CHUNK channel blocks.  (A variant of its own: in the common one the branches took 1 % of VGG-16.)
-template <int CG, bool LONG>
-__global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_constant__ Maps maps, const __grid_constant__ Params p) {
+template <int CG, bool LONG, bool ROWS8>
+__global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __grid_constant__ Maps maps, const __grid_constant__ Params p) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sbase = smem_u32(smem);
   auto full_a = [&](int s) { return sbase + 8u * s; };
@@ -69,6 +76,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
   int& s_refused = *reinterpret_cast<int*>(smem + 8 * BARS + 4);
   int& s_note = *reinterpret_cast<int*>(smem + 8 * BARS + 12);       // a result is not finite, see Note
   uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + 8 * BARS + 8);
+  int& s_plain = *reinterpret_cast<int*>(smem + 8 * BARS + 16);      // the blob holds no dense form
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const bool leader = CG == 1 || rank == 0;
@@ -77,12 +85,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
     s_abort = 0;
     s_refused = 0;
     s_note = 0;
+    if (ROWS8) s_plain = 0;
   }
-  if (threadIdx.x == W_A * 32) prefetch_map(&maps.a);
+  if (!ROWS8 && threadIdx.x == W_A * 32) prefetch_map(&maps.a);
   if (threadIdx.x == W_B * 32) prefetch_map(&maps.b);
   if (threadIdx.x < BARS) {                // a barrier each: 30 of them in a row by one thread showed in the launch
     const int t = (int)threadIdx.x, acc = t - (2 * MAX_A + 2 * MAX_B + 2);
-    const int count = acc == 0 || acc == 1 ? CG * EPI_WARPS : t == BARS - 3 ? EPI_WARPS : t == BARS - 2 ? p.parts : 1;
+    const int count = ROWS8 && t < MAX_A ? CG * ROW_WARPS : acc == 0 || acc == 1 ? CG * EPI_WARPS : t == BARS - 3 ? EPI_WARPS : t == BARS - 2 ? p.parts : 1;
     mbar_init(sbase + 8u * (uint32_t)t, (uint32_t)count);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -118,9 +127,74 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
     for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(bar, parity) && global_ns() - t0 <= p.wait_ns; ++spin) {}
   };
 
-  if (warp == W_A) {
+  if (ROWS8 && (warp == W_A || warp > W_MMA)) {
+    // =========================================================================== activations, in pieces of four channels
+    // The rows, their order and places are those of the TMA copies below; a warp takes every fourth row, 2, 4 or 8 positions at
+    // a time (as many pieces of each as the stage's channel steps read).  A stage is reported when the next one's copies have
+    // been issued, or when its slot is not free yet.  (What this costs is the latency of the address arithmetic: four copies
+    // are computed side by side.)
+    const int lw = warp == W_A ? 0 : warp - W_MMA;
+    const __half* x = static_cast<const __half*>(p.x);
+    int slot = 0, pending = -1;
+    uint32_t par = 1u;
+    auto report = [&](int s) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // before the tensor core reads them
+      __syncwarp();
+      if (lane == 0) {
+        if (CG == 2) arrive_remote(map_to_rank(full_a(s), 0u));
+        else mbar_arrive(full_a(s));
+      }
+    };
+    for (int item = unit; item < p.items && alive; item += n_units) {
+      const int tg = p.d_groups.div(item);
+      const int m0 = (CG == 2 ? 2 * tg + (int)rank : tg) * p.mstep;
+      const int v1 = p.d_P.div(m0), off = m0 - v1 * p.P, rows = p.d_P.div(off + p.ext) + 1;
+      for (int cb = cb0; cb < cb1 && alive; ++cb) {
+        const int ks = cb + 1 == p.ncb ? p.ks_last : KB / 16, lp = ks == 1 ? 2 : ks == 2 ? 3 : 4;     // 2^lp pieces of a position
+        const int piece = lane & ((1 << lp) - 1), i0 = lane >> lp, di = 32 >> lp, c = cb * KB + piece * 4;
+        for (int pl = 0; pl < p.planes; ++pl) {
+          const int dy = pl >> 1, dx = (pl & 1) - p.stride;
+          if (!__all_sync(0xFFFFFFFFu, mbar_try_wait(empty_a(slot), par))) {
+            if (pending >= 0) {
+              asm volatile("cp.async.wait_all;" ::: "memory");
+              report(pending);
+              pending = -1;
+            }
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait<20>(empty_a(slot), par, abort_flag, p.wait_ns))) { alive = false; break; }
+          }
+          const uint32_t row0 = sbase + OFF_RING + (uint32_t)slot * p.a_bytes;
+          for (int j = lw; j < rows; j += ROW_WARPS) {
+            const int v = v1 - 1 + j, vi = v < 0 ? 0 : p.d_HP.div(v), yr = v - vi * p.HP, n = p.d_strips.div(vi);
+            const int y = yr * p.stride + dy, x0 = (vi - n * p.strips) * p.Ws * p.stride + dx;
+            const bool row_in = yr >= 0 && y < p.H && n < p.N && c < p.C;
+            const __half* src = x + (((size_t)(row_in ? n : 0) * p.H + (row_in ? y : 0)) * p.W) * p.C + (row_in ? c : 0);
+            const uint32_t t0 = (uint32_t)(p.P - off + j * p.P), sub = ((uint32_t)piece & 1u) * 8u, chunk = (uint32_t)piece >> 1;
+            const int w = row_in ? p.W : 0;
+            for (int i = i0; i < p.P; i += 4 * di)
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int iu = i + u * di, xx = x0 + iu * p.stride;
+                const bool in = (unsigned)xx < (unsigned)w;
+                const uint32_t t = t0 + (uint32_t)iu, dst = row0 + t * 128u + ((chunk ^ (t & 7u)) << 4) + sub;
+                if (iu < p.P)
+                  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src + (in ? (ptrdiff_t)xx * p.C : 0)), "r"(in ? 8 : 0) : "memory");
+              }
+          }
+          asm volatile("cp.async.commit_group;" ::: "memory");
+          if (pending >= 0) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            report(pending);
+          }
+          pending = slot;
+          if (++slot == p.a_slots) { slot = 0; par ^= 1u; }
+        }
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (alive && pending >= 0) report(pending);
+  } else if (warp == W_A) {
     // =========================================================================== activations
-    if (elect_one()) {
+    if (!ROWS8 && elect_one()) {
       int slot = 0;
       uint32_t par = 1u, armed = 0u, armed_par = 0u;
       const uint32_t row_bytes = (uint32_t)p.P * 128u;
@@ -173,6 +247,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
     if (!blob_matches_warp(p)) {
       alive = false;
       if (lane == 0) { s_refused = 1; s_abort = 1; atomicExch(p.status, PAT_ERR_BLOB); }
+    } else if (ROWS8 && no_dense_form(p)) {
+      alive = false;
+      if (lane == 0) { s_refused = 1; s_plain = 1; s_abort = 1; }
     } else if (elect_one()) {
       int slot = 0, stage_no = 0;
       uint32_t par = 1u, armed = 0u, armed_par = 0u;
@@ -433,10 +510,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f16(const __grid_const
   if (failed && p.parts > 1) give_time();              // what the others had sent by then
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == W_MMA) free_columns<CG>(tmem);
-  if (s_note && !failed) {
+  if ((s_note && !failed) || (ROWS8 && s_plain)) {
     const bool whole = CG == 2 || p.parts == 1;
     renew_results<false, CG>(p, unit, n_units, CG == 2 ? (int)rank : 0, whole ? 0 : first_column<false>(p, (int)rank),
-                             whole ? p.BN : first_column<false>(p, (int)rank + 1));
+                             whole ? p.BN : first_column<false>(p, (int)rank + 1), ROWS8 && s_plain != 0);
   }
 }
 
@@ -494,13 +571,15 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   if (!dv) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cannot query the current device");
   Params p;
   using KernelFn = void (*)(const Maps, const Params);
-  static const KernelFn kernels[4] = {k_conv_mma_f16<1, false>, k_conv_mma_f16<2, false>, k_conv_mma_f16<1, true>, k_conv_mma_f16<2, true>};
+  static const KernelFn kernels[8] = {k_conv_mma_f16<1, false, false>, k_conv_mma_f16<2, false, false>, k_conv_mma_f16<1, true, false>, k_conv_mma_f16<2, true, false>,
+                                      k_conv_mma_f16<1, false, true>, k_conv_mma_f16<2, false, true>, k_conv_mma_f16<1, true, true>, k_conv_mma_f16<2, true, true>};
+  const bool rows8 = C % 8 != 0;
   static thread_local int at_once[kMaxDevices][4];
   const int di = (int)(dv - slots);
   if (!dv->ready) {
     for (KernelFn fn : kernels)
       if (int rc = check_cuda(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES), "set shared memory size")) return rc;
-    for (int i = 0; i < 4; ++i) at_once[di][i] = clusters_at_once(kernels[i == 1], 1 << i, NTHREADS, SMEM_BYTES);
+    for (int i = 0; i < 4; ++i) at_once[di][i] = clusters_at_once(kernels[i == 1], 1 << i, threads_of(false), SMEM_BYTES);
     dv->ready = true;
   }
   if (!set_geometry(p, TILE, N, H, W, stride, 0)) return set_error(PAT_ERR_SHAPE, "pat_conv3x3: too many tiles");
@@ -508,7 +587,7 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   if (act == 2 && !set_geometry(p, TILE, N, H, W, stride, 2)) return set_error(PAT_ERR_SHAPE, "pat_conv3x3: too many tiles");
   p.act = act;
   p.y = y;
-  set_packed(p, x, blob, L, F, K);
+  set_packed(p, x, blob, L, F, C, K);
   p.status = status_word();
   if (!p.status) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cannot resolve the status word");
   p.F = F; p.C = C; p.K = K; p.dtype = PAT_F16; p.n_keep = n_keep;
@@ -536,7 +615,7 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
 
   Maps maps;
   const cuuint32_t one[4] = {1, 1, 1, 1};
-  {
+  if (!rows8) {
     const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     const cuuint64_t pitch[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
     const cuuint32_t box[4] = {KB, (cuuint32_t)(stride * (p.P - 1) + 1), 1, 1}, step[4] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1};
@@ -560,9 +639,9 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   attr[1].val.clusterDim.x = sp.cg == 2 ? 2 : sp.parts; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 2;
-  cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.blockDim = dim3((unsigned)threads_of(rows8)); cfg.dynamicSmemBytes = SMEM_BYTES;
   cfg.gridDim = dim3((unsigned)(sp.parts > 1 ? p.items * sp.parts : sp.cg * std::min(p.items, at_once[di][sp.cg - 1])));
-  if (int rc = check_cuda(cudaLaunchKernelEx(&cfg, kernels[sp.cg - 1 + (p.ncb > CHUNK ? 2 : 0)], maps, p), "pat_conv3x3 launch")) return rc;
+  if (int rc = check_cuda(cudaLaunchKernelEx(&cfg, kernels[sp.cg - 1 + (p.ncb > CHUNK ? 2 : 0) + (rows8 ? 4 : 0)], maps, p), "pat_conv3x3 launch")) return rc;
   count_launches(1);
   return check_cuda(cudaGetLastError(), "pat_conv3x3 launch");
 }

@@ -43,6 +43,7 @@ struct Geometry {
   int* status;
   int N, H, W, F, C, K, dtype;
   long long n_keep;
+  unsigned long long dense_end;  // dense_form_end of the layer
   int Ho, Wo;                // output size before pooling
   int P, HP, Ws, strips;     // positions per row, rows per image (with its zero rows), columns and number of strips
   int tile_size, mstep;      // positions of a tile, positions from one tile to the next (whole row pairs when pooling)
@@ -221,6 +222,9 @@ __device__ __forceinline__ bool blob_matches_warp(const Geometry& p) {
   return __all_sync(0xFFFFFFFFu, ok) != 0;
 }
 
+// The blob holds no dense form, see dense_form_end: the results are formed from the packed kept taps alone.
+__device__ __forceinline__ bool no_dense_form(const Geometry& p) { return p.dense_end != 0 && p.hdr->total_bytes < p.dense_end; }
+
 // Output pixel of position m: index (n Ho + y) Wo + x, or -1 for padding positions.
 __device__ __forceinline__ int pixel_of(const Geometry& p, int m, int& y, int& x, int& n) {
   const int v = p.d_P.div(m), i = m - v * p.P;
@@ -311,9 +315,10 @@ __device__ __forceinline__ void store_one(const Geometry& p, size_t at, float v)
   if constexpr (F32) static_cast<float*>(p.y)[at] = v;
   else static_cast<__half*>(p.y)[at] = __float2half_rn(v);
 }
-// The results that this block has stored - columns c_begin to c_end of its items - gone over by all its warps.
+// The results that this block has stored - columns c_begin to c_end of its items - gone over by all its warps.  `all`: none has
+// been stored, every one is formed (layers without pooling only).
 template <bool F32, int CG>
-__device__ __noinline__ void renew_results(const Geometry& p, int unit, int n_units, int side, int c_begin, int c_end) {
+__device__ __noinline__ void renew_results(const Geometry& p, int unit, int n_units, int side, int c_begin, int c_end, bool all) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
   const int hw = p.Ws >> 1, n_out = p.act == 2 ? (p.d_P.div(p.mstep) >> 1) * hw : p.mstep;
   for (int item = unit; item < p.items; item += n_units) {
@@ -333,7 +338,7 @@ __device__ __noinline__ void renew_results(const Geometry& p, int unit, int n_un
         if (pixel < 0) continue;
         for (int f = f0 + lane; f < f1; f += 32) {
           const size_t at = (size_t)pixel * p.F + f;
-          const float old = stored<F32>(p.y, at);
+          const float old = all ? NAN : stored<F32>(p.y, at);
           if (old == old) continue;
           const float v = kept_taps<F32>(p, f, nn, yy, xx);
           store_one<F32>(p, at, p.act ? fmaxf(v, 0.0f) : v);       // (what pat_relu_maxpool makes of a NaN)
@@ -595,7 +600,8 @@ inline int set_exchange(Geometry& p, int per, int smem_bytes, int ring_at, int r
 }
 
 // Where the packed kernels are (see kept_taps).
-inline void set_packed(Geometry& p, const void* x, const void* blob, const BlobLayout& L, int F, int K) {
+inline void set_packed(Geometry& p, const void* x, const void* blob, const BlobLayout& L, int F, int C, int K) {
+  p.dense_end = dense_form_end(L, C);
   const char* b = static_cast<const char*>(blob);
   p.x = x;
   p.hdr = reinterpret_cast<const BlobHeader*>(b);

@@ -45,7 +45,7 @@ __host__ __device__ inline BlobPtrs blob_ptrs(void* blob, const BlobLayout& L, i
   p.tw4 = b + L.tw4;
   p.dboff = reinterpret_cast<uint32_t*>(b + L.dboff);
   p.dblk = b + L.dblk;
-  p.dense = L.scratch > L.dense ? reinterpret_cast<unsigned short*>(b + L.dense) : nullptr;
+  p.dense = L.dense ? reinterpret_cast<unsigned short*>(b + L.dense) : nullptr;
   p.hist = reinterpret_cast<int32_t*>(b + L.scratch);
   p.cnt = p.hist + (size_t)F * K;
   p.inv = reinterpret_cast<int32_t*>(b + inv_offset(L, F, K));
