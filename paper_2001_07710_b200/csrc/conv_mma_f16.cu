@@ -30,7 +30,7 @@
 // 41 us, 72 channels through TMA 25: the copies' issue bounds it).  These layers ran the generic multiply-add kernel before:
 // 28x28x260 -> 256, batch 32 508 -> 47 us, 9x10x212 -> 152, batch 8 255 -> 13, 80x81x20 -> 24, stride 2, batch 2 64 -> 16.
 //
-// Roles: warps 0-7 epilogue (tensor memory -> fp32 -> rectifier -> fp16 -> shared memory -> coalesced stores), warp 8
+// Roles: warps 0-7 epilogue (tensor memory -> fp32 -> rectifier -> fp16 -> whole sectors of the output; pooled through shared memory), warp 8
 // copies activations, warp 9 weights, warp 10 issues the multiply-adds (in the even CTA of a pair).  Every wait is
 // bounded; tensor memory is released on every path.
 #include "mma_tile.cuh"
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) {
-          if (CG == 2) arrive_remote(map_to_rank(acc_empty(buf), 0));
+          if (CG == 2) arrive_remote_read(map_to_rank(acc_empty(buf), 0));
           else mbar_arrive(acc_empty(buf));
         }
         if (++buf == n_acc) { buf = 0; pf ^= 1u; }
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           __syncwarp();
           if (lane == 0) {
-            if (CG == 2) arrive_remote(map_to_rank(acc_empty(buf), 0));
+            if (CG == 2) arrive_remote_read(map_to_rank(acc_empty(buf), 0));
             else mbar_arrive(acc_empty(buf));
           }
           if (CG == 2 && item + n_units >= p.items) { __syncwarp(); cluster_arrive(); left = true; }
@@ -479,9 +479,10 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
           float f[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) f[i] = max_nan(__uint_as_float(v[q][i]), floor_at);
-          stage_results<false>(row, sw, q, f);
+          if (p.act != 2) store_piece<false>(p, g * p.BN + c0 + q * 16, px < p.mstep ? pixel : -1, f, note);
+          else stage_results<false>(row, sw, q, f);
         }
-        store_results<false, 1>(p, st, g, c0, nc, pixel, m0, warp, lane, note);
+        if (p.act == 2) pool_results<false, 1>(p, st, g, c0, nc, m0, warp, lane, note);
       }
       if (++buf == n_acc) { buf = 0; pf ^= 1u; }
     }
@@ -587,6 +588,7 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   if (act == 2 && !set_geometry(p, TILE, N, H, W, stride, 2)) return set_error(PAT_ERR_SHAPE, "pat_conv3x3: too many tiles");
   p.act = act;
   p.y = y;
+  p.wide = aligned(y, 32) && F * 2 % 32 == 0;
   set_packed(p, x, blob, L, F, C, K);
   p.status = status_word();
   if (!p.status) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cannot resolve the status word");

@@ -48,6 +48,7 @@ struct alignas(64) Maps { CUtensorMap b; };
 struct Params : Geometry {
   int a_rows, a_slots;       // activations: rows of a part of a stage, ring slots
   uint32_t a_bytes;          // bytes of a slot (three parts)
+  int step_v, step_i;        // rows and columns from a position to the one A_ROWS / UNITS further on
 };
 
 __device__ __forceinline__ void load_b(int cg, uint32_t dst, const CUtensorMap* m, int c, int f, int t, uint32_t bar) {
@@ -105,16 +106,23 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
   auto locate = [&](int item) {
     const int m0 = (CG * p.d_groups.div(item) + (int)side) * p.mstep;
     valid = 0u;
+    // the first piece's position by divisions, the others by steps of 64 positions from it
+    const int q = m0 + t0, v1 = p.d_P.div(q), vi = v1 == 0 ? 0 : p.d_HP.div(v1 - 1);
+    int i = q - v1 * p.P, yr = v1 - 1 - vi * p.HP, n = p.d_strips.div(vi), strip = vi - n * p.strips;
 #pragma unroll
     for (int j = 0; j < UNITS; ++j) {
-      const int q = m0 + t0 + j * (A_ROWS / UNITS);
-      const int v1 = p.d_P.div(q), i = q - v1 * p.P, v = v1 - 1;
-      const int vi = v < 0 ? 0 : p.d_HP.div(v), yr = v - vi * p.HP, n = p.d_strips.div(vi), strip = vi - n * p.strips;
       const int y = yr * p.stride, x = (strip * p.Ws + i - 1) * p.stride;
       base[j] = (n * p.H + y) * p.W + x;
       if (t0 + j * (A_ROWS / UNITS) < rows && n < p.N && yr >= 0) {
         const uint32_t in_y = (y < p.H ? 3u : 0u) | (y + 1 < p.H ? 12u : 0u), x1 = x + 1;
         valid |= (in_y & ((x >= 0 && x < p.W ? 5u : 0u) | ((int)x1 >= 0 && (int)x1 < p.W ? 10u : 0u))) << (4 * j);
+      }
+      i += p.step_i;
+      yr += p.step_v;
+      if (i >= p.P) { i -= p.P; ++yr; }
+      while (yr >= p.HP) {
+        yr -= p.HP;
+        if (++strip == p.strips) { strip = 0; ++n; }
       }
     }
   };
@@ -129,7 +137,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
   if (threadIdx.x == W_B * 32) prefetch_map(&maps.b);
   if (threadIdx.x < BARS) {                // a barrier each: 30 of them in a row by one thread showed in the launch
     const int t = (int)threadIdx.x, acc = t - (2 * MAX_A + 2 * MAX_B + 2);
-    const int count = t < MAX_A ? CG * LOAD_WARPS : acc == 0 || acc == 1 ? CG * EPI_WARPS : t == BARS - 3 ? EPI_WARPS / 2 : t == BARS - 2 ? p.parts : 1;
+    const int count = t < MAX_A ? LOAD_WARPS + (CG == 2 && leader ? 1 : 0) : acc == 0 || acc == 1 ? CG * EPI_WARPS : t == BARS - 3 ? EPI_WARPS / 2 : t == BARS - 2 ? p.parts : 1;
     mbar_init(sbase + 8u * (uint32_t)t, (uint32_t)count);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -214,10 +222,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // before the tensor core reads them
           __syncwarp();
-          if (lane == 0) {
-            if (CG == 2) arrive_remote(map_to_rank(full_a(slot), pair));
-            else mbar_arrive(full_a(slot));
-          }
+          if (lane == 0) mbar_arrive(full_a(slot));
           if (++slot == p.a_slots) { slot = 0; par ^= 1u; }
         }
     }
@@ -326,6 +331,19 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
         else commit<1>(drain, 0u);
         let_land(drain, 0u);
       }
+    } else if (CG == 2) {
+      // The odd CTA's stages are reported to the even one by this warp, once each: an arrival on another CTA's barrier that
+      // passes on what was written before it waits for all of the thread's own accesses, which held the loading warps up (eight
+      // such arrivals a stage: 56x56x128 -> 128, stride 2, batch 32 61 us, 41 like this).
+      int sa = 0;
+      uint32_t pa = 0u;
+      for (int item = unit; item < p.items && alive; item += n_units)
+        for (int stage = (cb1 - cb0) * p.planes; stage > 0; --stage) {
+          if (!wait_warp(full_a(sa), pa, abort_flag, p.wait_ns)) { alive = false; break; }
+          if (lane == 0) arrive_remote(map_to_rank(full_a(sa), pair));
+          __syncwarp();
+          if (++sa == p.a_slots) { sa = 0; pa ^= 1u; }
+        }
     }
   } else if (warp < EPI_WARPS) {
     // =========================================================================== sums and results
@@ -354,20 +372,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           if (q * 16 < half) {
-            uint32_t v[16];
+            uint32_t v[16], w[16];
             tmem_load16(tc + (uint32_t)(BUF_COLS / 2 + q * 16), v);
+            tmem_load16(tc + (uint32_t)(q * 16), w);
             tile::tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) acc[q][i] += __uint_as_float(v[i]);
-            tmem_load16(tc + (uint32_t)(q * 16), v);
-            tile::tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) acc[q][i] += __uint_as_float(v[i]);
+            for (int i = 0; i < 16; ++i) acc[q][i] = (acc[q][i] + __uint_as_float(v[i])) + __uint_as_float(w[i]);
           }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) {
-          if (CG == 2) arrive_remote(map_to_rank(acc_empty(buf), pair));
+          if (CG == 2) arrive_remote_read(map_to_rank(acc_empty(buf), pair));
           else mbar_arrive(acc_empty(buf));
         }
         if (CG == 2 && c + 1 == n_chunks && item + n_units >= p.items) { __syncwarp(); cluster_arrive(); left = true; }
@@ -389,6 +404,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
         if (alive) add_parts<true, TILE, CG>(p, sbase, item, rank, note);
         break;
       }
+      if (p.act != 2) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q * 16 < half) {
+            float f[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) f[i] = max_nan(acc[q][i], floor_at);
+            store_piece<true>(p, g * p.BN + col0 + q * 16, pixel, f, note);
+          }
+        continue;
+      }
       const uint32_t row = st + (uint32_t)(warp * 32 + lane) * 128u, sw = (uint32_t)(lane & 7);
 #pragma unroll
       for (int h = 0; h < 2; ++h)
@@ -401,7 +427,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
               for (int i = 0; i < 16; ++i) f[i] = max_nan(acc[2 * h + q][i], floor_at);
               stage_results<true>(row, sw, q, f);
             }
-          store_results<true, 2>(p, st, g, col0 + h * 32, min(32, half - h * 32), pixel, m0, warp, lane, note);
+          pool_results<true, 2>(p, st, g, col0 + h * 32, min(32, half - h * 32), m0, warp, lane, note);
         }
     }
     if (note.taken()) s_note = 1;
@@ -516,6 +542,7 @@ int conv_mma_f32(const void* blob, int F, int C, const uint16_t* masks, int K, i
   if (act == 2 && !set_geometry(p, TILE, N, H, W, stride, 2)) return set_error(PAT_ERR_SHAPE, "pat_conv3x3: too many tiles");
   p.act = act;
   p.y = y;
+  p.wide = aligned(y, 32) && F * 4 % 32 == 0;
   set_packed(p, x, blob, L, F, C, K);
   p.status = status_word();
   if (!p.status) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cannot resolve the status word");
@@ -529,6 +556,8 @@ int conv_mma_f32(const void* blob, int F, int C, const uint16_t* masks, int K, i
   p.a_rows = (SUB + (stride == 2 ? p.P + 1 : 2 * p.P + 2) + 7) / 8 * 8;
   p.a_bytes = (uint32_t)(TERMS * p.a_rows) * 64u;
   p.a_bytes = (p.a_bytes + 1023) / 1024 * 1024;
+  p.step_v = A_ROWS / UNITS / p.P;
+  p.step_i = A_ROWS / UNITS % p.P;
   const int ring = set_exchange(p, kPer<true>, SMEM_BYTES, OFF_RING, RING_BYTES, (int)(2 * p.a_bytes + 3 * p.b_bytes));
   p.a_slots = std::max(2, std::min(MAX_A, (ring - 4 * (int)p.b_bytes) / (int)p.a_bytes));
   p.b_slots = std::min(MAX_B, (ring - p.a_slots * (int)p.a_bytes) / (int)p.b_bytes);

@@ -58,6 +58,7 @@ struct Geometry {
   int share;                 // columns that one part adds up, at most
   int handshake;             // that place overlaps the rings: its owner says when they are free
   int act;                   // 0, 1: rectifier, 2: rectifier and 2 x 2 max pooling
+  int wide;                  // rows of results start at multiples of 32 bytes
   int b_slots;               // ring slots of weights
   uint32_t b_bytes;          // bytes of one
   uint32_t idesc;
@@ -88,6 +89,11 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
 }
 __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// The same for a slot that has been read: nothing that this thread has written is passed on with it, so it need not wait until that is
+// seen by the cluster.
+__device__ __forceinline__ void arrive_remote_read(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // Sixteen bytes into another CTA's shared memory; they are counted on its barrier when they have arrived.
 __device__ __forceinline__ void store_async(uint32_t addr, const float4& v, uint32_t bar) {
@@ -370,34 +376,15 @@ __device__ __noinline__ void renew_results(const Geometry& p, int unit, int n_un
   }
 }
 
-// One pass of the epilogue: the results of up to 64 fp16 / 32 fp32 columns lie in the staging, 128 bytes per position
-// (16-byte chunks swizzled by the position's low bits), and leave as runs of 128 bytes of NHWC output.  HALVES = 2: warps
-// 4-7 hold other columns of the same 128 positions (in staging rows 128-255) instead of 128 more positions.
+// One pass of the epilogue with pooling: the results of up to 64 fp16 / 32 fp32 columns lie in the staging, 128 bytes per
+// position (16-byte chunks swizzled by the position's low bits), and leave as runs of 128 bytes of NHWC output.  HALVES = 2:
+// warps 4-7 hold other columns of the same 128 positions (in staging rows 128-255) instead of 128 more positions.
 template <bool F32, int HALVES>
-__device__ __forceinline__ void store_results(const Geometry& p, uint32_t st, int g, int c0, int nc, int pixel, int m0, int warp, int lane, Note& note) {
+__device__ __forceinline__ void pool_results(const Geometry& p, uint32_t st, int g, int c0, int nc, int m0, int warp, int lane, Note& note) {
   constexpr int PER = F32 ? 4 : 8;                     // values per 16-byte chunk
   const int q = lane & 7, f = g * p.BN + c0 + q * PER;
   const bool mine = q * PER < nc && f < p.F;
   char* y = static_cast<char*>(p.y);
-  if (p.act != 2) {
-    __syncwarp();
-    uint4 v[8];
-#pragma unroll
-    for (int it = 0; it < 8; ++it) {
-      const int r = it * 4 + (lane >> 3);
-      tile::lds128(st + (uint32_t)(warp * 32 + r) * 128u + (uint32_t)((q ^ (r & 7)) << 4), v[it].x, v[it].y, v[it].z, v[it].w);
-    }
-#pragma unroll
-    for (int it = 0; it < 8; ++it) {
-      const int px = __shfl_sync(0xFFFFFFFFu, pixel, it * 4 + (lane >> 3));
-      if (px >= 0 && mine) {
-        note.see<F32>(v[it]);
-        *reinterpret_cast<uint4*>(y + ((size_t)px * p.F + f) * (F32 ? 4 : 2)) = v[it];
-      }
-    }
-    __syncwarp();
-    return;
-  }
   // 2 x 2 max pooling: a tile is whole pairs of rows, so the four positions of a window lie in the staging
   asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
   const int hw = p.Ws >> 1, n_out = (p.d_P.div(p.mstep) >> 1) * hw, v0 = p.d_P.div(m0);
@@ -423,7 +410,39 @@ __device__ __forceinline__ void store_results(const Geometry& p, uint32_t st, in
   asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
 }
 
-// One 16-column piece of a position's results into the staging (see store_results).
+// One 16-column piece of this lane's position, straight from registers in 32-byte sectors (where rows start at multiples of them).
+// What a tile's end costs is the latency of its instructions, and through shared memory there were three times as many:
+// 188x188x32 -> 96, fp16, batch 5 22.4 -> 17.9 us, 28x28x128, batch 8 9.8 -> 9.2; fp32 84x88x16 -> 192, batch 36 138 -> 121.
+template <bool F32>
+__device__ __forceinline__ void store_piece(const Geometry& p, int f, int pixel, const float (&v)[16], Note& note) {
+  constexpr int WORDS = F32 ? 16 : 8, PER = F32 ? 4 : 8;
+  uint32_t w[WORDS];
+  if constexpr (F32) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(v[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = pack_f16(v[2 * i], v[2 * i + 1]);
+  }
+  if (pixel < 0 || f >= p.F) return;
+  char* y = static_cast<char*>(p.y) + ((size_t)pixel * p.F + f) * (F32 ? 4 : 2);
+  const int left = p.F - f;                            // a multiple of eight
+#pragma unroll
+  for (int i = 0; i < WORDS; i += 8) {
+    if (F32 && i / 8 * 8 >= left) break;
+    note.see<F32>(make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]));
+    note.see<F32>(make_uint4(w[i + 4], w[i + 5], w[i + 6], w[i + 7]));
+    if (p.wide && (F32 || left >= 16)) {
+      asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(y + 4 * i), "r"(w[i]), "r"(w[i + 1]), "r"(w[i + 2]), "r"(w[i + 3]),
+                   "r"(w[i + 4]), "r"(w[i + 5]), "r"(w[i + 6]), "r"(w[i + 7]) : "memory");
+    } else {
+      *reinterpret_cast<uint4*>(y + 4 * i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
+      if ((i + 4) * PER / 4 < left) *reinterpret_cast<uint4*>(y + 4 * i + 16) = make_uint4(w[i + 4], w[i + 5], w[i + 6], w[i + 7]);
+    }
+  }
+}
+
+// One 16-column piece of a position's results into the staging (see pool_results).
 template <bool F32>
 __device__ __forceinline__ void stage_results(uint32_t row, uint32_t sw, int q, const float (&f)[16]) {
   if constexpr (F32) {
