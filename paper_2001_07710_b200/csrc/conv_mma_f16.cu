@@ -51,7 +51,10 @@ constexpr int OFF_RING = 1024, RING_BYTES = 198656, OFF_ST = OFF_RING + RING_BYT
 static_assert(SMEM_BYTES <= 232448 && OFF_ST % 1024 == 0, "shared memory budget of one SM");
 static_assert(SMEM_BYTES - OFF_RING >= (128 + MAX_PARTS_MMA * kPer<false>) * TILE * 4, "the partial sums of 128 filters fit");
 
-struct alignas(64) Maps { CUtensorMap a, b; };
+struct alignas(64) Maps { CUtensorMap a, rows, b; };     // rows: ROWS image rows at a time
+// A tile is 7 (56 columns) to 35 (7 columns) image rows; one thread issues their copies, 50 clocks each, and with four rows in one
+// the first stage of 14x14 arrives 700 clocks sooner.  (Whole images at a time would not fit what is left of a slot.)
+constexpr int ROWS = 4;
 
 struct Params : Geometry {
   int a_slots;               // ring slots of activations
@@ -87,7 +90,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
     s_note = 0;
     if (ROWS8) s_plain = 0;
   }
-  if (!ROWS8 && threadIdx.x == W_A * 32) prefetch_map(&maps.a);
+  if (!ROWS8 && threadIdx.x == W_A * 32) { prefetch_map(&maps.a); prefetch_map(&maps.rows); }
   if (threadIdx.x == W_B * 32) prefetch_map(&maps.b);
   if (threadIdx.x < BARS) {                // a barrier each: 30 of them in a row by one thread showed in the launch
     const int t = (int)threadIdx.x, acc = t - (2 * MAX_A + 2 * MAX_B + 2);
@@ -96,6 +99,28 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == W_MMA) alloc_columns<CG>(smem_u32(&s_tmem));
+  const int unit = CG == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x / p.parts;
+  // Where an item's input rows are.  The tile's first position goes to row P of the slot, wherever it lies in its image row: both CTAs
+  // of a pair are addressed by the same descriptors.
+  struct Rows { int off, n_rows, y, strip, n; uint32_t bytes; };
+  auto find_rows = [&](int item) {
+    Rows r;
+    const int tg = p.d_groups.div(item);
+    const int m0 = (CG == 2 ? 2 * tg + (int)rank : tg) * p.mstep;
+    const int v1 = p.d_P.div(m0);
+    r.off = m0 - v1 * p.P;
+    r.n_rows = p.d_P.div(r.off + p.ext) + 1;
+    r.bytes = (uint32_t)(r.n_rows * p.P) * 128u;
+    if (CG == 2) {                           // and the other CTA's copies, which report here too (rank 0 arms the barrier)
+      const int m1 = m0 + p.mstep;
+      r.bytes += (uint32_t)((p.d_P.div(m1 - p.d_P.div(m1) * p.P + p.ext) + 1) * p.P) * 128u;
+    }
+    const int v0 = v1 - 1, vi = v0 < 0 ? 0 : p.d_HP.div(v0);
+    r.y = v0 - vi * p.HP;                    // -1 above the first image
+    r.n = p.d_strips.div(vi);
+    r.strip = vi - r.n * p.strips;
+    return r;
+  };
   // The other CTAs' barriers exist: a pair waits for that before its first copy, the parts of a layer before they send sums.
   // Blocks take a whole SM each, so most of a launch's blocks start when the kernel before it ends: what they do until
   // here is not hidden.
@@ -105,6 +130,8 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  Rows at = {};
+  if (!ROWS8 && warp == W_A) at = find_rows(unit);     // while the kernel before this one still runs
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (CG == 2) { cluster_wait(); met = true; }
@@ -115,7 +142,6 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
   // accumulator sets, beside the columns of the sums over several chunks
   const int sum_cols = LONG ? 2 * p.BN : 0, n_acc = 2 * 2 * p.BN + sum_cols <= (int)TMEM_COLS ? 2 : 1;
   // CG = 2: a pair walks over the items; CG = 1: a cluster of `parts` CTAs has one item, or single CTAs walk
-  const int unit = CG == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x / p.parts;
   const int n_units = CG == 2 ? (int)(gridDim.x >> 1) : (int)gridDim.x / p.parts;
   const int cb0 = CG == 2 ? 0 : (int)rank * p.ncb / p.parts;
   const int cb1 = CG == 2 ? p.ncb : ((int)rank + 1) * p.ncb / p.parts;
@@ -199,39 +225,35 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
       uint32_t par = 1u, armed = 0u, armed_par = 0u;
       const uint32_t row_bytes = (uint32_t)p.P * 128u;
       for (int item = unit; item < p.items && alive; item += n_units) {
-        const int tg = p.d_groups.div(item);
-        const int m0 = (CG == 2 ? 2 * tg + (int)rank : tg) * p.mstep;
-        // The tile's first position goes to row P of the slot, wherever it lies in its image row: both CTAs of a pair
-        // are addressed by the same descriptors.
-        const int v1 = p.d_P.div(m0), off = m0 - v1 * p.P, rows = p.d_P.div(off + p.ext) + 1;
-        uint32_t bytes = (uint32_t)rows * row_bytes;
-        if (CG == 2) {                       // and the other CTA's copies, which report here too (rank 0 arms the barrier)
-          const int m1 = m0 + p.mstep;
-          bytes += (uint32_t)(p.d_P.div(m1 - p.d_P.div(m1) * p.P + p.ext) + 1) * row_bytes;
-        }
-        const int v0 = v1 - 1;
-        const int vi0 = v0 < 0 ? 0 : p.d_HP.div(v0), y0 = v0 - vi0 * p.HP;     // y0 = -1 above the first image
-        const int n0 = p.d_strips.div(vi0), strip0 = vi0 - n0 * p.strips;
+        if (item != unit) at = find_rows(item);
         for (int cb = cb0; cb < cb1 && alive; ++cb)
           for (int pl = 0; pl < p.planes; ++pl) {
             const int dy = p.stride == 2 ? (pl >> 1) : 0, dx = (p.stride == 2 ? (pl & 1) : 0) - p.stride;
+            // fn(several, x, y, n): the rows from y on, as many of an image as there are at a time
+            auto each = [&](auto&& fn) {
+              int y = at.y, strip = at.strip, n = at.n;
+              for (int left = at.n_rows; left > 0;) {
+                const bool several = min(left, p.HP - y) >= ROWS;
+                fn(several, strip * p.Ws * p.stride + dx, y * p.stride + dy, n);
+                const int step = several ? ROWS : 1;
+                left -= step;
+                y += step;
+                if (y == p.HP) { y = 0; if (++strip == p.strips) { strip = 0; ++n; } }
+              }
+            };
             if (!mbar_try_wait(empty_a(slot), par)) {
               // the slot is still in use: bring the rows into L2 meanwhile
-              int y = y0, strip = strip0, n = n0;
-              for (int j = 0; j < rows; ++j) {
-                if (y >= 0 && y < p.Ho && n < p.N) prefetch_4d(&maps.a, cb * KB, strip * p.Ws * p.stride + dx, y * p.stride + dy, n);
-                if (++y == p.HP) { y = 0; if (++strip == p.strips) { strip = 0; ++n; } }
-              }
+              each([&](bool several, int x, int y, int n) {
+                if (y >= 0 && y < p.H && n < p.N) prefetch_4d(several ? &maps.rows : &maps.a, cb * KB, x, y, n);
+              });
               if (!mbar_wait<20>(empty_a(slot), par, abort_flag, p.wait_ns)) { alive = false; break; }
             }
-            if (leader) mbar_arrive_expect_tx(full_a(slot), bytes);
-            uint32_t dst = sbase + OFF_RING + (uint32_t)slot * p.a_bytes + (uint32_t)(p.P - off) * 128u;
-            int y = y0, strip = strip0, n = n0;
-            for (int j = 0; j < rows; ++j) {
-              load_4d<CG>(dst, &maps.a, cb * KB, strip * p.Ws * p.stride + dx, y * p.stride + dy, n, full_a(slot));
-              dst += row_bytes;
-              if (++y == p.HP) { y = 0; if (++strip == p.strips) { strip = 0; ++n; } }
-            }
+            if (leader) mbar_arrive_expect_tx(full_a(slot), at.bytes);
+            uint32_t dst = sbase + OFF_RING + (uint32_t)slot * p.a_bytes + (uint32_t)(p.P - at.off) * 128u;
+            each([&](bool several, int x, int y, int n) {
+              load_4d<CG>(dst, several ? &maps.rows : &maps.a, cb * KB, x, y, n, full_a(slot));
+              dst += several ? ROWS * row_bytes : row_bytes;
+            });
             armed |= 1u << slot;
             armed_par = (armed_par & ~(1u << slot)) | ((par ^ 1u) << slot);
             if (++slot == p.a_slots) { slot = 0; par ^= 1u; }
@@ -620,10 +642,13 @@ int conv_mma_f16(const void* blob, int F, int C, const uint16_t* masks, int K, i
   if (!rows8) {
     const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     const cuuint64_t pitch[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-    const cuuint32_t box[4] = {KB, (cuuint32_t)(stride * (p.P - 1) + 1), 1, 1}, step[4] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1};
-    const CUresult r = encode_fn()(&maps.a, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(x), dims, pitch, box, step,
-                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cuTensorMapEncodeTiled failed (%d)", (int)r);
+    const cuuint32_t step[4] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1};
+    for (int rows : {1, ROWS}) {
+      const cuuint32_t box[4] = {KB, (cuuint32_t)(stride * (p.P - 1) + 1), (cuuint32_t)(stride * (rows - 1) + 1), 1};
+      const CUresult r = encode_fn()(rows == 1 ? &maps.a : &maps.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(x), dims, pitch, box, step,
+                                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS) return set_error(PAT_ERR_CUDA, "pat_conv3x3: cuTensorMapEncodeTiled failed (%d)", (int)r);
+    }
   }
   {
     const cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)F, 9};

@@ -219,12 +219,27 @@ __device__ __forceinline__ int axis_taps(int stride, int odd) { return stride ==
 __device__ __forceinline__ int axis_tap(int stride, int odd, int k) { return stride == 1 ? k : (odd ? 2 * k : 1); }
 __device__ __forceinline__ int axis_shift(int stride, int odd, int k) { return stride == 1 ? k : (odd ? k : 1); }
 
-// The blob was packed with the parameters of this call (one warp; the same answer in every lane).
+// The blob was packed with the parameters of this call (one warp; the same answer in every lane).  A word of the header and masks
+// per lane, read side by side: the first weights wait for this.
 __device__ __forceinline__ bool blob_matches_warp(const Geometry& p) {
+  const int lane = threadIdx.x & 31;
   const BlobHeader* bh = p.hdr;
-  bool ok = bh->magic == kBlobMagic && bh->version == kBlobVersion && bh->F == p.F && bh->C == p.C &&
-            bh->K == p.K && bh->dtype == p.dtype && bh->n_keep == p.n_keep;
-  for (int j = threadIdx.x & 31; j < p.K; j += 32) ok = ok && bh->masks[j] == p.masks[j];
+  static_assert(offsetof(BlobHeader, version) == 4 && offsetof(BlobHeader, F) == 8 && offsetof(BlobHeader, C) == 12 && offsetof(BlobHeader, K) == 16 &&
+                offsetof(BlobHeader, dtype) == 20 && offsetof(BlobHeader, n_keep) == 24, "the header's first eight words");
+  uint32_t word = 0u, want = 0u, mask = 0u, want_mask = 0u;
+  if (lane < 8) word = reinterpret_cast<const uint32_t*>(bh)[lane];
+  if (lane < p.K) mask = bh->masks[lane];
+  if (lane == 0) want = kBlobMagic;
+  if (lane == 1) want = kBlobVersion;
+  if (lane == 2) want = (uint32_t)p.F;
+  if (lane == 3) want = (uint32_t)p.C;
+  if (lane == 4) want = (uint32_t)p.K;
+  if (lane == 5) want = (uint32_t)p.dtype;
+  if (lane == 6) want = (uint32_t)p.n_keep;
+  if (lane == 7) want = (uint32_t)((unsigned long long)p.n_keep >> 32);
+  if (lane < p.K) want_mask = p.masks[lane];
+  bool ok = word == want && mask == want_mask;
+  for (int j = lane + 32; j < p.K; j += 32) ok = ok && bh->masks[j] == p.masks[j];
   return __all_sync(0xFFFFFFFFu, ok) != 0;
 }
 
