@@ -27,23 +27,41 @@ __device__ __forceinline__ uint4 relu_max(uint4 a, uint4 b, bool f16) {
   return r;
 }
 
-// chunks: 16-byte chunks per pixel (C * element size / 16).  One thread per (output pixel, chunk), chunks fastest.
-template <bool POOL>
-__global__ void __launch_bounds__(256) k_relu_maxpool(const uint4* __restrict__ x, uint4* __restrict__ y, long long n_out,
-                                                      int Ho, int Wo, int W, int chunks, bool f16) {
+// chunks: 16-byte chunks per pixel (C * element size / 16).  One thread per (output pixel, chunk), chunks fastest, from the last one
+// down: what the kernel before this one wrote last is still in L2 when the tensor is larger than that, and so is what the next one
+// reads first.  Bound by the bytes when large, by the launch when small: a dependent launch, and divisions by multiplication
+// (Index = unsigned; long long beyond 2^31 chunks).  Convolution and pooling together: 12x20x32 -> 448, one image 8.5 -> 7.0 us,
+// 188x188x32 -> 96, batch 5 23.9 -> 21.1, 32x32x128, batch 128 33.6 -> 32.2.
+struct PoolSizes {
+  int Wo, W, chunks;
+  FastDiv d_Wo, d_chunks;
+};
+template <bool POOL, typename Index>
+__global__ void __launch_bounds__(256) k_relu_maxpool(const uint4* x, uint4* y, long long n_out, PoolSizes p, bool f16) {
+  pdl_wait();
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_out; t += stride) {
-    const int ck = (int)(t % chunks);
-    const long long px = t / chunks;                         // (n, yo, xo) flattened
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += stride) {
+    const long long t = n_out - 1 - i;
     if (!POOL) {
       const uint4 v = __ldcs(x + t);
       __stcs(y + t, relu_max(v, v, f16));
     } else {
-      const int xo = (int)(px % Wo);
-      const long long row = px / Wo;                         // n * Ho + yo  ->  input row 2 * row (H = 2 Ho)
-      const long long i00 = ((2 * row) * W + 2 * xo) * chunks + ck;
-      const uint4 a = __ldcs(x + i00), b = __ldcs(x + i00 + chunks);
-      const uint4 c = __ldcs(x + i00 + (long long)W * chunks), d = __ldcs(x + i00 + (long long)W * chunks + chunks);
+      long long row;                                         // n * Ho + yo  ->  input row 2 * row (H = 2 Ho)
+      int ck, xo;
+      if constexpr (sizeof(Index) == 4) {
+        const int px = p.d_chunks.div((int)t), r = p.d_Wo.div(px);      // (n, yo, xo) flattened
+        ck = (int)t - px * p.chunks;
+        xo = px - r * p.Wo;
+        row = r;
+      } else {
+        const long long px = t / p.chunks;
+        ck = (int)(t % p.chunks);
+        row = px / p.Wo;
+        xo = (int)(px % p.Wo);
+      }
+      const long long i00 = ((2 * row) * p.W + 2 * xo) * p.chunks + ck;
+      const uint4 a = __ldcs(x + i00), b = __ldcs(x + i00 + p.chunks);
+      const uint4 c = __ldcs(x + i00 + (long long)p.W * p.chunks), d = __ldcs(x + i00 + (long long)p.W * p.chunks + p.chunks);
       __stcs(y + t, relu_max(relu_max(a, b, f16), relu_max(c, d, f16), f16));
     }
   }
@@ -51,8 +69,8 @@ __global__ void __launch_bounds__(256) k_relu_maxpool(const uint4* __restrict__ 
 
 // Any channel count (no 16-byte chunks): one thread per output element.
 template <typename T>
-__global__ void __launch_bounds__(256) k_relu_maxpool_scalar(const T* __restrict__ x, T* __restrict__ y, long long n_out,
-                                                             int Ho, int Wo, int W, int C, int pool) {
+__global__ void __launch_bounds__(256) k_relu_maxpool_scalar(const T* x, T* y, long long n_out, int Wo, int W, int C, int pool) {
+  pdl_wait();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_out; t += stride) {
     const int c = (int)(t % C);
@@ -88,15 +106,20 @@ extern "C" int pat_relu_maxpool(const void* x, int dtype, int N, int H, int W, i
   const long long n_out = (long long)N * Ho * Wo * (vec ? (C * elem / 16) : C);
   const long long blocks = (n_out + 255) / 256;
   const unsigned grid = (unsigned)(blocks < 148 * 64 ? blocks : 148 * 64);   // grid-stride beyond that
+  cudaError_t e;
   if (vec) {
-    const int chunks = C * elem / 16;
-    if (pool) k_relu_maxpool<true><<<grid, 256, 0, st>>>(static_cast<const uint4*>(x), static_cast<uint4*>(y), n_out, Ho, Wo, W, chunks, dtype == PAT_F16);
-    else k_relu_maxpool<false><<<grid, 256, 0, st>>>(static_cast<const uint4*>(x), static_cast<uint4*>(y), n_out, Ho, Wo, W, chunks, dtype == PAT_F16);
+    PoolSizes p;
+    p.Wo = Wo; p.W = W; p.chunks = C * elem / 16;
+    p.d_Wo.set(Wo); p.d_chunks.set(p.chunks);
+    const bool small = n_out <= 0x7FFFFFFFll;
+    e = launch_dependent(!pool ? k_relu_maxpool<false, unsigned> : small ? k_relu_maxpool<true, unsigned> : k_relu_maxpool<true, long long>, dim3(grid), dim3(256), 0, st,
+                         static_cast<const uint4*>(x), static_cast<uint4*>(y), n_out, p, dtype == PAT_F16);
   } else if (dtype == PAT_F16) {
-    k_relu_maxpool_scalar<__half><<<grid, 256, 0, st>>>(static_cast<const __half*>(x), static_cast<__half*>(y), n_out, Ho, Wo, W, C, pool);
+    e = launch_dependent(k_relu_maxpool_scalar<__half>, dim3(grid), dim3(256), 0, st, static_cast<const __half*>(x), static_cast<__half*>(y), n_out, Wo, W, C, pool);
   } else {
-    k_relu_maxpool_scalar<float><<<grid, 256, 0, st>>>(static_cast<const float*>(x), static_cast<float*>(y), n_out, Ho, Wo, W, C, pool);
+    e = launch_dependent(k_relu_maxpool_scalar<float>, dim3(grid), dim3(256), 0, st, static_cast<const float*>(x), static_cast<float*>(y), n_out, Wo, W, C, pool);
   }
+  if (e != cudaSuccess) return check_cuda(e, "pat_relu_maxpool launch");
   count_launches(1);
   return check_cuda(cudaGetLastError(), "pat_relu_maxpool launch");
 }

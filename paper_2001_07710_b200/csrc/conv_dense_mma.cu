@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_conv_dense_c3_mma(const Args a)
   __shared__ __align__(16) __half tile[(TH + 2) * ROWP];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
+  pdl_wait();
 
   // weight fragments: k-step q, n-tile jt: b0 = B[k = 16 q + 2t, 2t + 1][n = g], b1 = B[k = 16 q + 2t + 8, 2t + 9][n = g],
   // with B[k = 9 r + 3 s + c][n] = w[channel_of(jt, n)][c][r][s] for k < 27 and zero above
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_conv_dense_c3_mma(const Args a)
 #pragma unroll
     for (int jt = 0; jt < 8; ++jt) {
       const float* wf = a.w + (size_t)channel_of(jt, g) * 27;
-      auto wk = [&](int k) { return k < 27 ? __float2half_rn(__ldg(wf + 9 * (k % 3) + k / 3)) : __float2half_rn(0.0f); };
+      auto wk = [&](int k) { return k < 27 ? __float2half_rn(wf[9 * (k % 3) + k / 3]) : __float2half_rn(0.0f); };
       bw[q][jt][0] = pack2(wk(16 * q + 2 * t), wk(16 * q + 2 * t + 1));
       bw[q][jt][1] = pack2(wk(16 * q + 2 * t + 8), wk(16 * q + 2 * t + 9));
     }
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_conv_dense_c3_mma(const Args a)
         const int yy = ty * TH - 1 + row, xx = tx * TW - 1 + (j == RW - 1 ? TW + 1 : (2 * j) / 3);
         if (i < WIN && yy >= 0 && yy < a.H && xx >= 0 && xx < a.W) {
           const long long h0 = (((long long)n * a.H + yy) * a.W + tx * TW - 1) * 3 - 1;   // even: the row's first word
-          win[q] = __ldg(reinterpret_cast<const uint32_t*>(a.x + h0) + j);
+          win[q] = reinterpret_cast<const uint32_t*>(a.x + h0)[j];
         }
       } else {
         const int row = i / ((TW + 2) * 3), rem = i % ((TW + 2) * 3);
@@ -183,8 +184,8 @@ int conv_dense_c3_mma(const float* w, const void* x, void* y, int N, int H, int 
   const int sm_count = dv->sms;
   const long long want = (long long)sm_count * 8;         // eight resident blocks of four warps per SM
   const unsigned grid = (unsigned)(a.n_tiles < want ? a.n_tiles : want);
-  if (W % 2 == 0) k_conv_dense_c3_mma<true><<<grid, NTHREADS, 0, st>>>(a);
-  else k_conv_dense_c3_mma<false><<<grid, NTHREADS, 0, st>>>(a);
+  const cudaError_t e = launch_dependent(W % 2 == 0 ? k_conv_dense_c3_mma<true> : k_conv_dense_c3_mma<false>, dim3(grid), dim3(NTHREADS), 0, st, a);
+  if (e != cudaSuccess) return check_cuda(e, "pat_conv3x3_dense launch");
   count_launches(1);
   return check_cuda(cudaGetLastError(), "pat_conv3x3_dense launch");
 }

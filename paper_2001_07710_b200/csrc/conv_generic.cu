@@ -311,6 +311,7 @@ __global__ void __launch_bounds__(256, 2) k_conv_dense_c3_f32(DenseArgs a, long 
   constexpr int ROW = (TW + 2) * 3, WIN = (TH + 2) * ROW, PER = (WIN + 255) / 256;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, fg = lane & 7, px0 = 8 * (lane >> 3);
   const int f0 = (int)blockIdx.y * 64;
+  pdl_wait();
   for (int i = t; i < 64 * 27; i += 256) s_w[i % 27][i / 27] = a.w[(size_t)f0 * 27 + i];
   const float* x = static_cast<const float*>(a.x);
   float win[PER];
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(256, 2) k_conv_dense_c3_f32(DenseArgs a, long 
     for (int q = 0; q < PER; ++q) {
       const int i = t + q * 256, row = i / ROW, e = i % ROW;
       const int yy = ty * TH - 1 + row, xx = tx * TW - 1 + e / 3;
-      win[q] = i < WIN && yy >= 0 && yy < a.H && xx >= 0 && xx < a.W ? __ldg(x + (((size_t)n * a.H + yy) * a.W + tx * TW - 1) * 3 + e) : 0.0f;
+      win[q] = i < WIN && yy >= 0 && yy < a.H && xx >= 0 && xx < a.W ? x[(((size_t)n * a.H + yy) * a.W + tx * TW - 1) * 3 + e] : 0.0f;
     }
   };
   if ((long long)blockIdx.x < n_tiles) load_window(blockIdx.x);
@@ -457,7 +458,8 @@ extern "C" int pat_conv3x3_dense(const float* w, int F, int C, int dtype, const 
     DeviceSlot* dv = device_slot(slots);
     if (!dv) return set_error(PAT_ERR_CUDA, "pat_conv3x3_dense: cannot query the current device");
     const long long n_tiles = (long long)N * a.tiles_x * a.tiles_y, most = 2ll * dv->sms;
-    k_conv_dense_c3_f32<<<dim3((unsigned)(n_tiles < most ? n_tiles : most), (unsigned)(F / 64)), 256, 0, st>>>(a, n_tiles);
+    const cudaError_t e = launch_dependent(k_conv_dense_c3_f32, dim3((unsigned)(n_tiles < most ? n_tiles : most), (unsigned)(F / 64)), dim3(256), 0, st, a, n_tiles);
+    if (e != cudaSuccess) return check_cuda(e, "pat_conv3x3_dense launch");
     count_launches(1);
     return check_cuda(cudaGetLastError(), "pat_conv3x3_dense launch");
   }
