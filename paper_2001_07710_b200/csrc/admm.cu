@@ -41,6 +41,7 @@ constexpr int kVecQ = 16;
 template <int L>
 __global__ void __launch_bounds__(32 * kVecWarps, 5) k_simplex_project(const float* d, long long n, int K, float* u) {
   constexpr int G = 32 / L;                // vectors per warp
+  pdl_wait();
   const int lane = threadIdx.x & 31, sl = lane & (L - 1), g = lane / L;
   const long long stride = (long long)gridDim.x * kVecWarps * G;
   const long long first = ((long long)blockIdx.x * kVecWarps + (threadIdx.x >> 5)) * G;
@@ -62,16 +63,19 @@ __global__ void __launch_bounds__(32 * kVecWarps, 5) k_simplex_project(const flo
     for (int q = 1; q < kVecQ; ++q) top = fmaxf(top, x[q]);
     float nu32 = (group_sum<L>(top) - 1.0f) / (float)L;
     if (!(nu32 > -3.402823466e38f)) nu32 = -3.402823466e38f;   // overflow of the sum (or a NaN): start below every entry
-    // Counts are kept as floats (exact up to 2^24): a pass is then one comparison and two predicated additions per entry.
+    // Counts are kept as floats (exact up to 2^24): a pass is then one comparison and one predicated addition of a pair, the entry
+    // and a one, per entry.
+    unsigned long long pair[kVecQ];
+#pragma unroll
+    for (int q = 0; q < kVecQ; ++q) pair[q] = 0x3F80000000000000ull | __float_as_uint(x[q]);
     float before = -1.0f;
     bool done = false;
     for (int round = 0; round < K + 2; ++round) {       // fp32 rounds
-      float s = 0.0f, c = 0.0f;
+      unsigned long long sc = 0ull;
 #pragma unroll
       for (int q = 0; q < kVecQ; ++q)
-        if (x[q] > nu32) { s += x[q]; c += 1.0f; }
-      s = group_sum<L>(s);
-      c = group_sum<L>(c);
+        asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p add.rn.f32x2 %0, %0, %3;\n\t}" : "+l"(sc) : "f"(x[q]), "f"(nu32), "l"(pair[q]));
+      const float s = group_sum<L>(__uint_as_float((unsigned)sc)), c = group_sum<L>(__uint_as_float((unsigned)(sc >> 32)));
       if (!done) {
         if (c == before || c == 0.0f) { done = true; before = c; }   // the set repeats (or rounding has pushed nu past the largest entry)
         else { nu32 = (s - 1.0f) / c; before = c; }
@@ -133,11 +137,12 @@ __device__ __forceinline__ unsigned ordered(float v) {    // unsigned order = or
 }
 // Q: entries per lane of a warp that shares a vector (0: K <= 32, a thread per vector)
 template <int Q>
-__global__ void __launch_bounds__(kBinThreads) k_argmax_binarize(const float* __restrict__ z, long long n, int K, int per_tile, FastDiv d_K,
-                                                                 unsigned char* __restrict__ index_out, float* __restrict__ onehot_out) {
+__global__ void __launch_bounds__(kBinThreads) k_argmax_binarize(const float* z, long long n, int K, int per_tile, FastDiv d_K,
+                                                                 unsigned char* index_out, float* onehot_out) {
   __shared__ __align__(16) float s_z[kBinFloats];
   __shared__ uint8_t s_best[kBinFloats];
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  pdl_wait();
   for (long long i0 = (long long)blockIdx.x * per_tile; i0 < n; i0 += (long long)gridDim.x * per_tile) {
     const int m = (int)(n - i0 < per_tile ? n - i0 : per_tile), e = m * K;
     const float* src = z + i0 * K;
@@ -224,13 +229,13 @@ __global__ void __launch_bounds__(kBinThreads) k_argmax_binarize(const float* __
 // one is its programmatic dependent and does everything but the last additions before it waits for it.
 // FULL: the library is all 126 masks, so the best one holds the four largest squares (the whole call at 262144
 // kernels: 67 -> 10.5 us; a loop over 56 masks takes 21.5, so smaller libraries do not need a search of their own).
-constexpr int kAssignThreads = 256, kAssignPerThread = 2, kFullK = 126;
+constexpr int kAssignThreads = 256, kFullK = 126;
 __global__ void __launch_bounds__(256) k_zero_counts(unsigned long long* counts, int K) {
   pdl_wait();
   if ((int)threadIdx.x < K) counts[threadIdx.x] = 0ull;
 }
 template <bool FULL>
-__global__ void __launch_bounds__(kAssignThreads) k_assign_count(const float* __restrict__ w, long long n, MaskTable lib,
+__global__ void __launch_bounds__(kAssignThreads) k_assign_count(const float* __restrict__ w, long long n, int rounds, MaskTable lib,
                                                                  unsigned long long* __restrict__ counts) {
   __shared__ unsigned int s_cnt[kMaxK + 1];
   __shared__ uint8_t s_id[FULL ? 512 : 1];                  // mask -> library id
@@ -238,8 +243,8 @@ __global__ void __launch_bounds__(kAssignThreads) k_assign_count(const float* __
   const int t = threadIdx.x;
   for (int q = t; q <= kMaxK; q += kAssignThreads) s_cnt[q] = 0u;
   if (FULL && t < kFullK) s_id[lib.m[t]] = (uint8_t)t;
-  for (int r = 0; r < kAssignPerThread; ++r) {
-    const long long i0 = ((long long)blockIdx.x * kAssignPerThread + r) * kAssignThreads;
+  for (int r = 0; r < rounds; ++r) {
+    const long long i0 = ((long long)blockIdx.x * rounds + r) * kAssignThreads;
     __syncthreads();
     if (i0 >= n) break;
     const int m = (int)((n - i0 < kAssignThreads ? n - i0 : kAssignThreads) * 9);
@@ -322,11 +327,10 @@ extern "C" int pat_simplex_project(const float* d, int64_t n, int K, float* u, v
   if (!aligned(d, 4) || !aligned(u, 4)) return set_error(PAT_ERR_ALIGN, "pat_simplex_project: buffers must be 4-byte aligned");
   if (n == 0) return PAT_OK;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (K <= 16) k_simplex_project<1><<<vec_grid(n, 32), 32 * kVecWarps, 0, st>>>(d, (long long)n, K, u);
-  else if (K <= 32) k_simplex_project<2><<<vec_grid(n, 16), 32 * kVecWarps, 0, st>>>(d, (long long)n, K, u);
-  else if (K <= 64) k_simplex_project<4><<<vec_grid(n, 8), 32 * kVecWarps, 0, st>>>(d, (long long)n, K, u);
-  else if (K <= 128) k_simplex_project<8><<<vec_grid(n, 4), 32 * kVecWarps, 0, st>>>(d, (long long)n, K, u);
-  else k_simplex_project<16><<<vec_grid(n, 2), 32 * kVecWarps, 0, st>>>(d, (long long)n, K, u);
+  const auto fn = K <= 16 ? k_simplex_project<1> : K <= 32 ? k_simplex_project<2> : K <= 64 ? k_simplex_project<4> : K <= 128 ? k_simplex_project<8> : k_simplex_project<16>;
+  const int per_warp = K <= 16 ? 32 : K <= 32 ? 16 : K <= 64 ? 8 : K <= 128 ? 4 : 2;
+  const cudaError_t e = launch_dependent(fn, dim3(vec_grid(n, per_warp)), dim3(32 * kVecWarps), 0, st, d, (long long)n, K, u);
+  if (e != cudaSuccess) return check_cuda(e, "pat_simplex_project launch");
   count_launches(1);
   return check_cuda(cudaGetLastError(), "pat_simplex_project launch");
 }
@@ -349,7 +353,8 @@ extern "C" int pat_argmax_binarize(const float* z, int64_t n, int K, uint8_t* in
   d_K.set(K);
   const long long tiles = (n + per_tile - 1) / per_tile;
   const auto fn = K <= 32 ? k_argmax_binarize<0> : K <= 64 ? k_argmax_binarize<2> : K <= 128 ? k_argmax_binarize<4> : k_argmax_binarize<8>;
-  fn<<<(unsigned)(tiles < most ? tiles : most), kBinThreads, 0, st>>>(z, (long long)n, K, per_tile, d_K, index_out, onehot_out);
+  const cudaError_t e = launch_dependent(fn, dim3((unsigned)(tiles < most ? tiles : most)), dim3(kBinThreads), 0, st, z, (long long)n, K, per_tile, d_K, index_out, onehot_out);
+  if (e != cudaSuccess) return check_cuda(e, "pat_argmax_binarize launch");
   count_launches(1);
   return check_cuda(cudaGetLastError(), "pat_argmax_binarize launch");
 }
@@ -369,9 +374,11 @@ extern "C" int pat_extract_library(const float* w, int64_t n, const uint16_t* ma
   cudaError_t le = launch_dependent(k_zero_counts, dim3(1), dim3(256), 0, st, counts, K_in);
   count_launches(1);
   if (n > 0 && le == cudaSuccess) {
-    const unsigned grid = (unsigned)((n + kAssignThreads * kAssignPerThread - 1) / (kAssignThreads * kAssignPerThread));
+    // two kernels a thread, so that a block adds its counts up once for 512 of them; one when that leaves the chip idle
+    const int rounds = n > 148 * 8 * kAssignThreads ? 2 : 1;
+    const unsigned grid = (unsigned)((n + kAssignThreads * rounds - 1) / (kAssignThreads * rounds));
     // 126 distinct masks of four entries are all there are
-    le = launch_dependent(K_in == kFullK ? k_assign_count<true> : k_assign_count<false>, dim3(grid), dim3(kAssignThreads), 0, st, w, (long long)n, lib, counts);
+    le = launch_dependent(K_in == kFullK ? k_assign_count<true> : k_assign_count<false>, dim3(grid), dim3(kAssignThreads), 0, st, w, (long long)n, rounds, lib, counts);
     count_launches(1);
   }
   if (le == cudaSuccess)
