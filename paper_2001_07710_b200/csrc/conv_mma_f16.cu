@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
             if (CG == 2) arrive_remote_read(map_to_rank(acc_empty(buf), 0));
             else mbar_arrive(acc_empty(buf));
           }
-          if (CG == 2 && item + n_units >= p.items) { __syncwarp(); cluster_arrive(); left = true; }
+          if (CG == 2 && item + n_units >= p.items) { cluster_arrive(); left = true; }
         }
         const uint32_t row = st + (uint32_t)px * 128u, sw = (uint32_t)(px & 7);
 #pragma unroll

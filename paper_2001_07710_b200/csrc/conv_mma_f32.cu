@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
           if (CG == 2) arrive_remote_read(map_to_rank(acc_empty(buf), pair));
           else mbar_arrive(acc_empty(buf));
         }
-        if (CG == 2 && c + 1 == n_chunks && item + n_units >= p.items) { __syncwarp(); cluster_arrive(); left = true; }
+        if (CG == 2 && c + 1 == n_chunks && item + n_units >= p.items) { cluster_arrive(); left = true; }
         if (++buf == 2) { buf = 0; pf ^= 1u; }
       }
       if (p.act == 2 || p.parts > 1) alive = all_epilogue_warps(alive);         // they meet at barriers below: all go on or none

@@ -79,9 +79,19 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+// Instructions marked .aligned are undefined in a warp whose lanes have parted, and only __syncwarp() promises that they have met
+// again behind a branch that they did not all take.  The ones that run a few times a launch begin with it; for those on tensor
+// memory, store_piece and send_part, whose branches precede them, end with it.
+
 // The two halves of a barrier of the whole cluster (threads that have exited count as arrived).
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
@@ -157,6 +167,7 @@ __device__ __forceinline__ void commit(uint32_t bar, uint32_t pair) {
 }
 template <int CG>
 __device__ __forceinline__ void alloc_columns(uint32_t smem_dst) {
+  __syncwarp();
   if constexpr (CG == 2) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "n"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -167,6 +178,7 @@ __device__ __forceinline__ void alloc_columns(uint32_t smem_dst) {
 }
 template <int CG>
 __device__ __forceinline__ void free_columns(uint32_t taddr) {
+  __syncwarp();
   if constexpr (CG == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(TMEM_COLS) : "memory");
   else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(TMEM_COLS) : "memory");
 }
@@ -422,6 +434,7 @@ __device__ __forceinline__ void pool_results(const Geometry& p, uint32_t st, int
       for (int k = 0; k < 4; ++k) note.see<F32>(w[k]);
     if (keep) *reinterpret_cast<uint4*>(y + ((((size_t)n * (p.Ho >> 1) + (yy >> 1)) * (p.Wo >> 1) + (xx >> 1)) * p.F + f) * (F32 ? 4 : 2)) = m;
   }
+  __syncwarp();
   asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
 }
 
@@ -439,22 +452,24 @@ __device__ __forceinline__ void store_piece(const Geometry& p, int f, int pixel,
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = pack_f16(v[2 * i], v[2 * i + 1]);
   }
-  if (pixel < 0 || f >= p.F) return;
-  char* y = static_cast<char*>(p.y) + ((size_t)pixel * p.F + f) * (F32 ? 4 : 2);
-  const int left = p.F - f;                            // a multiple of eight
+  if (pixel >= 0 && f < p.F) {
+    char* y = static_cast<char*>(p.y) + ((size_t)pixel * p.F + f) * (F32 ? 4 : 2);
+    const int left = p.F - f;                            // a multiple of eight
 #pragma unroll
-  for (int i = 0; i < WORDS; i += 8) {
-    if (F32 && i / 8 * 8 >= left) break;
-    note.see<F32>(make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]));
-    note.see<F32>(make_uint4(w[i + 4], w[i + 5], w[i + 6], w[i + 7]));
-    if (p.wide && (F32 || left >= 16)) {
-      asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(y + 4 * i), "r"(w[i]), "r"(w[i + 1]), "r"(w[i + 2]), "r"(w[i + 3]),
-                   "r"(w[i + 4]), "r"(w[i + 5]), "r"(w[i + 6]), "r"(w[i + 7]) : "memory");
-    } else {
-      *reinterpret_cast<uint4*>(y + 4 * i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
-      if ((i + 4) * PER / 4 < left) *reinterpret_cast<uint4*>(y + 4 * i + 16) = make_uint4(w[i + 4], w[i + 5], w[i + 6], w[i + 7]);
+    for (int i = 0; i < WORDS; i += 8) {
+      if (F32 && i / 8 * 8 >= left) break;
+      note.see<F32>(make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]));
+      note.see<F32>(make_uint4(w[i + 4], w[i + 5], w[i + 6], w[i + 7]));
+      if (p.wide && (F32 || left >= 16)) {
+        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(y + 4 * i), "r"(w[i]), "r"(w[i + 1]), "r"(w[i + 2]), "r"(w[i + 3]),
+                     "r"(w[i + 4]), "r"(w[i + 5]), "r"(w[i + 6]), "r"(w[i + 7]) : "memory");
+      } else {
+        *reinterpret_cast<uint4*>(y + 4 * i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
+        if ((i + 4) * PER / 4 < left) *reinterpret_cast<uint4*>(y + 4 * i + 16) = make_uint4(w[i + 4], w[i + 5], w[i + 6], w[i + 7]);
+      }
     }
   }
+  __syncwarp();                                        // positions of padding store nothing
 }
 
 // One 16-column piece of a position's results into the staging (see pool_results).
@@ -503,6 +518,7 @@ __device__ __forceinline__ void send_part(const Geometry& p, uint32_t sbase, uin
       store_async(map_to_rank(at, to), w, map_to_rank(bar, to));
     }
   }
+  __syncwarp();                                        // positions of padding send nothing
 }
 // This CTA's share, by the epilogue's warps, in the order of the channels.
 template <bool F32, int T, int CG>

@@ -401,8 +401,9 @@ constexpr int kSelThreads = 1024, kSelList = 3328, kSelFew = 128, kSelBlocks = 8
 constexpr int64_t kBlockKeys = 16384, kClusterKeys = 131072;
 template <int R>
 __device__ __forceinline__ void sel_barrier() {
-  if constexpr (R == 1) __syncthreads();
-  else asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if constexpr (R == 1) { __syncthreads(); return; }
+  __syncwarp();                                      // (.aligned, behind branches that lanes take apart)
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Address of a block's shared memory, and what is done there.
 __device__ __forceinline__ uint32_t sel_addr(const void* p, uint32_t rank) {
