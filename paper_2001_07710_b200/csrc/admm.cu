@@ -36,10 +36,12 @@ __device__ __forceinline__ T group_sum(T v) {
 //
 // L lanes share a vector, sixteen entries each (K <= 16 L), so a warp works on 32 / L vectors at once: a round is a
 // chain of dependent steps (a sum over the group, a division, a comparison), and what the kernel needs is many such
-// chains in flight, not many lanes per chain.  Entry j of a vector sits in lane j % L, slot j / L.  u may be d.
+// chains in flight, not many lanes per chain.  Entry j of a vector sits in lane j % L, slot j / L.  u may be d.  A thread that
+// has a vector to itself exchanges nothing and wants registers for it rather than a fifth block per SM (131072 x 16: 16.1 ->
+// 13.7 us, 262144 x 12: 17.7 -> 16.9).
 constexpr int kVecQ = 16;
 template <int L>
-__global__ void __launch_bounds__(32 * kVecWarps, 5) k_simplex_project(const float* d, long long n, int K, float* u) {
+__global__ void __launch_bounds__(32 * kVecWarps, L == 1 ? 4 : 5) k_simplex_project(const float* d, long long n, int K, float* u) {
   constexpr int G = 32 / L;                // vectors per warp
   pdl_wait();
   const int lane = threadIdx.x & 31, sl = lane & (L - 1), g = lane / L;
@@ -63,19 +65,18 @@ __global__ void __launch_bounds__(32 * kVecWarps, 5) k_simplex_project(const flo
     for (int q = 1; q < kVecQ; ++q) top = fmaxf(top, x[q]);
     float nu32 = (group_sum<L>(top) - 1.0f) / (float)L;
     if (!(nu32 > -3.402823466e38f)) nu32 = -3.402823466e38f;   // overflow of the sum (or a NaN): start below every entry
-    // Counts are kept as floats (exact up to 2^24): a pass is then one comparison and one predicated addition of a pair, the entry
-    // and a one, per entry.
-    unsigned long long pair[kVecQ];
-#pragma unroll
-    for (int q = 0; q < kVecQ; ++q) pair[q] = 0x3F80000000000000ull | __float_as_uint(x[q]);
+    // Counts are kept as floats (exact up to 2^24): a pass is then one comparison and two predicated additions per entry.  (One
+    // addition of a pair, the entry and a one, wants 32 registers where these take 16, and spilled 32 - 40 bytes: 262144 vectors
+    // of 126, 56 and 24 entries took 74.8, 42.8 and 21.3 us; 63.7, 35.0 and 19.1 like this.)
     float before = -1.0f;
     bool done = false;
     for (int round = 0; round < K + 2; ++round) {       // fp32 rounds
-      unsigned long long sc = 0ull;
+      float s = 0.0f, c = 0.0f;
 #pragma unroll
       for (int q = 0; q < kVecQ; ++q)
-        asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p add.rn.f32x2 %0, %0, %3;\n\t}" : "+l"(sc) : "f"(x[q]), "f"(nu32), "l"(pair[q]));
-      const float s = group_sum<L>(__uint_as_float((unsigned)sc)), c = group_sum<L>(__uint_as_float((unsigned)(sc >> 32)));
+        if (x[q] > nu32) { s += x[q]; c += 1.0f; }
+      s = group_sum<L>(s);
+      c = group_sum<L>(c);
       if (!done) {
         if (c == before || c == 0.0f) { done = true; before = c; }   // the set repeats (or rounding has pushed nu past the largest entry)
         else { nu32 = (s - 1.0f) / c; before = c; }
