@@ -235,8 +235,11 @@ __global__ void __launch_bounds__(256) k_zero_counts(unsigned long long* counts,
   pdl_wait();
   if ((int)threadIdx.x < K) counts[threadIdx.x] = 0ull;
 }
-template <bool FULL>
-__global__ void __launch_bounds__(kAssignThreads) k_assign_count(const float* __restrict__ w, long long n, int rounds, MaskTable lib,
+// ROUNDS: kernels of a thread.  With one, twice as many blocks end and add their counts to the same few lines: for the full library, whose
+// blocks are short, that costs more than it gives once all SMs have several (262144 kernels 16.6 us, 11.8 with two; 196608 13.0,
+// 10.4; but 163840 8.9, 10.0 and 4096 6.6, 7.7).  Smaller libraries: one (262144 kernels, 56 masks 18.8, 22.3 with two; 12 masks 8.5, 9.1).
+template <bool FULL, int ROUNDS>
+__global__ void __launch_bounds__(kAssignThreads) k_assign_count(const float* __restrict__ w, long long n, MaskTable lib,
                                                                  unsigned long long* __restrict__ counts) {
   __shared__ unsigned int s_cnt[kMaxK + 1];
   __shared__ uint8_t s_id[FULL ? 512 : 1];                  // mask -> library id
@@ -244,8 +247,8 @@ __global__ void __launch_bounds__(kAssignThreads) k_assign_count(const float* __
   const int t = threadIdx.x;
   for (int q = t; q <= kMaxK; q += kAssignThreads) s_cnt[q] = 0u;
   if (FULL && t < kFullK) s_id[lib.m[t]] = (uint8_t)t;
-  for (int r = 0; r < rounds; ++r) {
-    const long long i0 = ((long long)blockIdx.x * rounds + r) * kAssignThreads;
+  for (int r = 0; r < ROUNDS; ++r) {
+    const long long i0 = ((long long)blockIdx.x * ROUNDS + r) * kAssignThreads;
     __syncthreads();
     if (i0 >= n) break;
     const int m = (int)((n - i0 < kAssignThreads ? n - i0 : kAssignThreads) * 9);
@@ -375,11 +378,14 @@ extern "C" int pat_extract_library(const float* w, int64_t n, const uint16_t* ma
   cudaError_t le = launch_dependent(k_zero_counts, dim3(1), dim3(256), 0, st, counts, K_in);
   count_launches(1);
   if (n > 0 && le == cudaSuccess) {
-    // two kernels a thread, so that a block adds its counts up once for 512 of them; one when that leaves the chip idle
-    const int rounds = n > 148 * 8 * kAssignThreads ? 2 : 1;
+    // 126 distinct masks of four entries are all there are; two kernels a thread from two and a half blocks per SM on (see k_assign_count)
+    static thread_local DeviceSlot slots[kMaxDevices];
+    DeviceSlot* dv = device_slot(slots);
+    const bool full = K_in == kFullK;
+    const int rounds = full && 2 * ((n + 2 * kAssignThreads - 1) / (2 * kAssignThreads)) >= 5ll * (dv ? dv->sms : 148) ? 2 : 1;
+    const auto fn = !full ? k_assign_count<false, 1> : rounds == 1 ? k_assign_count<true, 1> : k_assign_count<true, 2>;
     const unsigned grid = (unsigned)((n + kAssignThreads * rounds - 1) / (kAssignThreads * rounds));
-    // 126 distinct masks of four entries are all there are
-    le = launch_dependent(K_in == kFullK ? k_assign_count<true> : k_assign_count<false>, dim3(grid), dim3(kAssignThreads), 0, st, w, (long long)n, rounds, lib, counts);
+    le = launch_dependent(fn, dim3(grid), dim3(kAssignThreads), 0, st, w, (long long)n, lib, counts);
     count_launches(1);
   }
   if (le == cudaSuccess)
