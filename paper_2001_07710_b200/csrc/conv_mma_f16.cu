@@ -189,22 +189,41 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
             if (!__all_sync(0xFFFFFFFFu, mbar_wait<20>(empty_a(slot), par, abort_flag, p.wait_ns))) { alive = false; break; }
           }
           const uint32_t row0 = sbase + OFF_RING + (uint32_t)slot * p.a_bytes;
-          for (int j = lw; j < rows; j += ROW_WARPS) {
-            const int v = v1 - 1 + j, vi = v < 0 ? 0 : p.d_HP.div(v), yr = v - vi * p.HP, n = p.d_strips.div(vi);
-            const int y = yr * p.stride + dy, x0 = (vi - n * p.strips) * p.Ws * p.stride + dx;
-            const bool row_in = yr >= 0 && y < p.H && n < p.N && c < p.C;
-            const __half* src = x + (((size_t)(row_in ? n : 0) * p.H + (row_in ? y : 0)) * p.W) * p.C + (row_in ? c : 0);
-            const uint32_t t0 = (uint32_t)(p.P - off + j * p.P), sub = ((uint32_t)piece & 1u) * 8u, chunk = (uint32_t)piece >> 1;
-            const int w = row_in ? p.W : 0;
-            for (int i = i0; i < p.P; i += 4 * di)
+          // Narrow images: what counts is the number of rows that a warp goes through, one after the other, most of its lanes idle.
+          // There the lanes take positions of any row, which costs three divisions a piece (400 7x7x36, stride 2, 64 filters 19 -> 23
+          // us: so only below).  4 -> 64, us, rows and positions: 1x1 16.5, 6.2, stride 2 50.6, 9.5; 7x7 8.3, 6.4; 28x28 6.5, 6.9.
+          if (2 * p.P <= 5 * di) {
+            const int total = rows * p.P;
+            for (int e0 = 4 * di * lw + i0; e0 < total; e0 += ROW_WARPS * 4 * di)
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
-                const int iu = i + u * di, xx = x0 + iu * p.stride;
-                const bool in = (unsigned)xx < (unsigned)w;
-                const uint32_t t = t0 + (uint32_t)iu, dst = row0 + t * 128u + ((chunk ^ (t & 7u)) << 4) + sub;
-                if (iu < p.P)
-                  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src + (in ? (ptrdiff_t)xx * p.C : 0)), "r"(in ? 8 : 0) : "memory");
+                const int e = e0 + u * di, j = p.d_P.div(e), i = e - j * p.P;
+                const int v = v1 - 1 + j, vi = v < 0 ? 0 : p.d_HP.div(v), yr = v - vi * p.HP, n = p.d_strips.div(vi);
+                const int y = yr * p.stride + dy, xx = ((vi - n * p.strips) * p.Ws + i) * p.stride + dx;
+                const bool in = yr >= 0 && y < p.H && n < p.N && c < p.C && (unsigned)xx < (unsigned)p.W;
+                const uint32_t t = (uint32_t)(p.P - off + e), dst = row0 + t * 128u + ((((uint32_t)piece >> 1) ^ (t & 7u)) << 4) + ((uint32_t)piece & 1u) * 8u;
+                if (e < total)
+                  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;"
+                               ::"r"(dst), "l"(x + (in ? (size_t)((n * p.H + y) * p.W + xx) * p.C + c : 0)), "r"(in ? 8 : 0) : "memory");
               }
+          } else {
+            for (int j = lw; j < rows; j += ROW_WARPS) {
+              const int v = v1 - 1 + j, vi = v < 0 ? 0 : p.d_HP.div(v), yr = v - vi * p.HP, n = p.d_strips.div(vi);
+              const int y = yr * p.stride + dy, x0 = (vi - n * p.strips) * p.Ws * p.stride + dx;
+              const bool row_in = yr >= 0 && y < p.H && n < p.N && c < p.C;
+              const __half* src = x + (((size_t)(row_in ? n : 0) * p.H + (row_in ? y : 0)) * p.W) * p.C + (row_in ? c : 0);
+              const uint32_t t0 = (uint32_t)(p.P - off + j * p.P), sub = ((uint32_t)piece & 1u) * 8u, chunk = (uint32_t)piece >> 1;
+              const int w = row_in ? p.W : 0;
+              for (int i = i0; i < p.P; i += 4 * di)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const int iu = i + u * di, xx = x0 + iu * p.stride;
+                  const bool in = (unsigned)xx < (unsigned)w;
+                  const uint32_t t = t0 + (uint32_t)iu, dst = row0 + t * 128u + ((chunk ^ (t & 7u)) << 4) + sub;
+                  if (iu < p.P)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src + (in ? (ptrdiff_t)xx * p.C : 0)), "r"(in ? 8 : 0) : "memory");
+                }
+            }
           }
           asm volatile("cp.async.commit_group;" ::: "memory");
           if (pending >= 0) {

@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import paper_2001_07710_b200 as pc
+from timing import graph_ms
 
 pytestmark = pytest.mark.gpu
 
@@ -35,23 +36,8 @@ def test_counts_next_to_the_line(off, K):
 
 def test_a_smaller_layer_takes_no_longer():
     """A kernel a thread in a layer of 512 x 512 took half as long again as two: more than a layer of a sixth more kernels."""
-    def us(n):
+    def ms(n):
         w, counts, out = weights(n), torch.empty(126, dtype=torch.int64, device="cuda"), torch.empty(12, dtype=torch.int16, device="cuda")
-        call = lambda: pc.pat_extract_library(w, MASKS, 12, masks_out=out, counts=counts)
-        call()
-        stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
-        stream.wait_stream(torch.cuda.current_stream())
-        with torch.cuda.graph(graph, stream=stream):
-            for _ in range(20):
-                call()
-        times = []
-        for _ in range(9):
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            graph.replay()
-            b.record()
-            b.synchronize()
-            times.append(a.elapsed_time(b))
-        return sorted(times)[4]
-    us(512 * 512)
-    assert us(512 * 512) <= 1.25 * us(303105)              # measured 11.8 and 11.0 us; 16.6 and 11.1 with one
+        return graph_ms(lambda: pc.pat_extract_library(w, MASKS, 12, masks_out=out, counts=counts))
+    ms(512 * 512)
+    assert ms(512 * 512) <= 1.25 * ms(303105)              # measured 11.8 and 11.0 us; 16.6 and 11.1 with one
