@@ -74,7 +74,7 @@ __device__ inline int best_mask_fast(const float* __restrict__ wk, const MaskTab
   float best32 = -1.0f, second32 = -1.0f;
   int best = 0;
   bool plain = true;                       // every fp32 energy is an ordinary finite number
-#pragma unroll 4
+#pragma unroll 4                           // (projection of 512 x 512 kernels, 126 masks: 62.8 -> 60.5 us)
   for (int j = 0; j < lib.K; ++j) {
     const unsigned m = lib.m[j];
     float e = 0.0f;
