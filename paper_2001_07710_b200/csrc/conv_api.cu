@@ -46,7 +46,28 @@ static int check_conv_args(const void* blob, int F, int C, const uint16_t* masks
   return PAT_OK;
 }
 
-static bool on_tensor_cores(int F, int C, int dtype, int N, int H, int W, int stride) {
+// Odd multiples of four channels so few that a stage of the tensor-core kernels is mostly empty, with few filters: large images are
+// faster in the generic kernel, which pays by the kept kernel.  In fp32 its rows of 8 - 40 bytes of weights, read by all SMs at once,
+// lie in a few lines of L2 on top of that.  fp32, four patterns, generic and tensor cores, us:
+//   8 x 256x256, 4 -> 8 keep 1 67, 175, 4 -> 32 keep 0.3 115, 167 (keep 1 133, 160), 4 -> 40 keep 0.1 149, 202 (keep 1 186, 168), 4 -> 64 205, 137
+//   12 -> 8 keep 0.3 65, 78, 12 -> 16 keep 0.1 67, 97 (0.3 84, 79), 12 -> 24 keep 0.1 87, 79, 20 -> 8 keep 0.1 82, 110 (0.3 103, 103)
+//   2 x 256x256, 4 -> 16 keep 0.3 29, 29, 4 -> 24 34, 33, 4 -> 32 43, 46; 8 x 112x112, 4 -> 8 20, 26, 4 -> 16 23, 23, 4 -> 40 36, 44, one image 4 -> 8 10, 9; stride 2, 24 x 224x224, 4 -> 8 keep 0.3 68, 81, 4 -> 16
+//   keep 0.1 70, 78 (0.3 75, 74), 8 x 112x112 18, 13
+// (a rectifier behind the generic kernel, a pass of its own, adds 2 - 20 us)
+// fp16: 24 x 224x224, 12 -> 8 keep 0.02 100, 116, 0.3 no difference.
+static bool few_channels(int F, int C, int64_t n_keep, int dtype, int N, int H, int W, int stride) {
+  if (C % 8 == 0 || C > 20) return false;
+  const long long positions = (long long)N * ((H - 1) / stride + 1) * ((W - 1) / stride + 1);
+  const bool sparse = 8 * n_keep <= (int64_t)F * C;
+  if (dtype == PAT_F16) return stride == 1 && C <= 12 && F == 8 && sparse && positions >= 500000;
+  const bool large = positions >= 250000, third = 3 * n_keep <= (int64_t)F * C;
+  if (stride == 2) return positions >= 130000 && C <= 12 && (F == 8 ? C == 4 || sparse : C == 4 && F <= 16 && sparse);
+  if (C == 4) return F == 8 ? positions >= 20000 : (F <= 32 && large) || (F > 24 && F <= 40 && third && positions >= 90000);
+  return positions >= 130000 && ((sparse && F <= (C == 12 ? 16 : 8)) || (C == 12 && F == 8 && large && third));
+}
+
+static bool on_tensor_cores(int F, int C, int64_t n_keep, int dtype, int N, int H, int W, int stride) {
+  if (few_channels(F, C, n_keep, dtype, N, H, W, stride)) return false;
   return dtype == PAT_F16 ? conv_mma_f16_supported(F, C, dtype, N, H, W, stride) : conv_mma_f32_supported(F, C, dtype, N, H, W, stride);
 }
 static int conv_mma(const void* blob, int F, int C, const uint16_t* masks, int K, int64_t n_keep, int dtype, const void* x, void* y,
@@ -72,7 +93,7 @@ extern "C" int pat_conv3x3(const void* blob, int F, int C, const uint16_t* masks
                            int dtype, const void* x, void* y, int N, int H, int W, int stride, void* stream) {
   if (int rc = check_conv_args(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride)) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (on_tensor_cores(F, C, dtype, N, H, W, stride)) return conv_mma(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride, 0, stream);
+  if (on_tensor_cores(F, C, n_keep, dtype, N, H, W, stride)) return conv_mma(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride, 0, stream);
   return conv_generic(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride, st);
 }
 
@@ -101,7 +122,7 @@ extern "C" int pat_conv3x3_ws_act(const void* blob, int F, int C, const uint16_t
     if (prefer_img(F, C, masks, K, n_keep, dtype, N, H, W, stride))
       return conv_f32_img(blob, F, C, masks, K, n_keep, x, y, N, H, W, act, workspace, reinterpret_cast<cudaStream_t>(stream));
   }
-  if (on_tensor_cores(F, C, dtype, N, H, W, stride)) return conv_mma(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride, act, stream);
+  if (on_tensor_cores(F, C, n_keep, dtype, N, H, W, stride)) return conv_mma(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride, act, stream);
   if (act == 2) return set_error(PAT_ERR_SHAPE, "pat_conv3x3_ws_act: image too large");
   // the plain convolution, then the rectifier in place
   if (int rc = pat_conv3x3(blob, F, C, masks, K, n_keep, dtype, x, y, N, H, W, stride, stream)) return rc;

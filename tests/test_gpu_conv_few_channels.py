@@ -1,0 +1,36 @@
+"""Layers of few channels and filters: an odd multiple of four channels, where the generic kernel runs them on large images."""
+import pytest
+import torch
+
+import paper_2001_07710_b200 as pc
+from test_gpu_conv_mma import check
+from timing import graph_ms
+
+pytestmark = pytest.mark.gpu
+
+
+# both sides of the lines: positions, filters, kept kernels
+@pytest.mark.parametrize("dtype", ["f16", "f32"])
+@pytest.mark.parametrize("case", [
+    (2, 100, 100, 4, 8, 4, 1.0, 1, 0), (2, 100, 99, 4, 8, 4, 1.0, 1, 0),
+    (5, 250, 200, 4, 16, 4, 1.0, 1, 1), (5, 250, 199, 4, 16, 4, 1.0, 1, 1), (8, 250, 200, 4, 32, 8, 0.75, 1, 0),
+    (1, 300, 301, 4, 40, 8, 0.3, 1, 1), (1, 300, 301, 4, 40, 8, 0.5, 1, 1), (1, 300, 301, 4, 48, 8, 0.3, 1, 0),
+    (3, 210, 210, 12, 16, 8, 0.125, 1, 1), (3, 210, 210, 12, 24, 8, 0.125, 1, 0), (2, 256, 256, 20, 8, 12, 0.1, 1, 0), (2, 256, 256, 20, 8, 12, 0.3, 1, 0),
+    (2, 511, 512, 4, 8, 8, 0.5, 2, 1), (2, 511, 512, 4, 16, 8, 0.125, 2, 1), (2, 511, 512, 12, 8, 8, 0.1, 2, 0), (8, 250, 250, 12, 8, 8, 0.1, 1, 1),
+], ids=lambda c: "-".join(str(v) for v in c))
+def test_conv(case, dtype):
+    check(case, dtype)
+
+
+@pytest.mark.parametrize("N,H,F,stride", [(8, 256, 8, 1), (8, 256, 16, 1), (24, 224, 8, 2)])
+def test_four_channels_take_no_longer_than_six(N, H, F, stride):
+    """Six take the generic kernel.  Measured with a quarter of the kernels kept: 8 x 256x256 -> 8 53 us here, 116 on the tensor cores."""
+    def ms(C):
+        masks, n_keep = pc.pat_library_builtin(4), F * C // 4
+        pid, wm = pc.pat_project(torch.ones((F, C, 3, 3), device="cuda"), masks, n_keep)
+        blob = pc.pat_pack(wm, pid, masks, n_keep, "f32")
+        x = torch.ones((N, H, H, C), device="cuda")
+        y = pc.pat_conv3x3(blob, F, C, masks, n_keep, "f32", x, stride)
+        return graph_ms(lambda: pc.pat_conv3x3(blob, F, C, masks, n_keep, "f32", x, stride, y=y), calls=10)
+    ms(4)
+    assert ms(4) <= 1.1 * ms(6)
