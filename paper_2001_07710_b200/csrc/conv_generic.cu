@@ -8,19 +8,14 @@
 // channels at a time from NHWC global memory into a channel-planar fp32 shared-memory tile with its halo
 // (zero outside the image), so each activation is read from global memory once per block.  Only the four
 // stored taps of every kept kernel are visited (Section 6.2: per-pattern access, pattern-grouped kernels).
-#include "common.cuh"
+#include "plain_tile.cuh"
 
 namespace pat {
 namespace {
 
-constexpr int TH = 8, TW = 32, NWARP = 8, RF = 4, FG = NWARP * RF, CB = kChanTile;
+using namespace plain;
 
-template <typename T> __device__ inline float to_f32(T v);
-template <> __device__ inline float to_f32<float>(float v) { return v; }
-template <> __device__ inline float to_f32<__half>(__half v) { return __half2float(v); }
-template <typename T> __device__ inline T from_f32(float v);
-template <> __device__ inline float from_f32<float>(float v) { return v; }
-template <> __device__ inline __half from_f32<__half>(float v) { return __float2half_rn(v); }
+constexpr int NWARP = 8, FG = NWARP * RF;
 
 struct ConvArgs {
   const void* x;
@@ -34,13 +29,6 @@ struct ConvArgs {
   int N, H, W, C, F, Ho, Wo, K, nct, dtype;
   long long n_keep;
   int tiles_x, tiles_y;
-};
-
-template <int STRIDE> struct Geo {
-  static constexpr int IH = (TH - 1) * STRIDE + 3;
-  static constexpr int IW = (TW - 1) * STRIDE + 3;
-  static constexpr int IWP = IW | 1;                 // odd row pitch
-  static constexpr int PLANE = IH * IWP + ((IH * IWP) % 2 == 0 ? 1 : 0);   // odd plane pitch
 };
 
 // Stage channels [c0, c0+CB) of the input tile into shared memory as fp32, channel-planar.

@@ -48,7 +48,7 @@ constexpr int MAX_A = 4, MAX_B = 8;             // ring slots
 constexpr int CHUNK = 8;                        // channel blocks in one sum of the tensor core
 constexpr int ST_BYTES = TILE * 128;            // epilogue staging: 128 bytes per position
 constexpr int OFF_RING = 1024, RING_BYTES = 198656, OFF_ST = OFF_RING + RING_BYTES, SMEM_BYTES = OFF_ST + ST_BYTES;
-static_assert(SMEM_BYTES <= 232448 && OFF_ST % 1024 == 0, "shared memory budget of one SM");
+static_assert(SMEM_BYTES <= 232448 && OFF_ST % 1024 == 0 && OFF_RING == RING_AT && SMEM_BYTES == RING_TO, "shared memory budget of one SM");
 static_assert(SMEM_BYTES - OFF_RING >= (128 + MAX_PARTS_MMA * kPer<false>) * TILE * 4, "the partial sums of 128 filters fit");
 
 struct alignas(64) Maps { CUtensorMap a, rows, b; };     // rows: ROWS image rows at a time
@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
     // are computed side by side.)
     const int lw = warp == W_A ? 0 : warp - W_MMA;
     const __half* x = static_cast<const __half*>(p.x);
+    const uint64_t blob_bytes = p.hdr->total_bytes;     // looked at when the first copies have been issued
     int slot = 0, pending = -1;
     uint32_t par = 1u;
     auto report = [&](int s) {
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
           }
           pending = slot;
           if (++slot == p.a_slots) { slot = 0; par ^= 1u; }
+          if (blob_bytes < p.dense_end) { alive = false; break; }
         }
       }
     }
@@ -334,6 +336,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
     // The whole warp runs the loop with warp-uniform values and control flow (so that the operands' descriptors stay in
     // uniform registers) and one elected lane issues.  What the loop costs beside the multiply-adds shows: the tensor core
     // takes a tap's eight of them in 360 clocks at 64 filters; as one thread's loop they were issued in 640.
+    if (ROWS8) alive = __all_sync(0xFFFFFFFFu, !no_dense_form(p)) != 0;
     if (leader) {
       const bool el = elect_one();
       int sa = 0, sb = 0, buf = 0;
@@ -430,6 +433,7 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     Note note;
     const float floor_at = p.act != 0 ? 0.0f : -INFINITY;       // the rectifier
+    if (ROWS8) alive = __all_sync(0xFFFFFFFFu, !no_dense_form(p)) != 0;
     for (int item = unit; item < p.items && alive; item += n_units) {
       const int tg = p.d_groups.div(item), g = item - tg * p.groups;
       const int m0 = (CG == 2 ? 2 * tg + (int)rank : tg) * p.mstep;
@@ -523,30 +527,29 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
     }
     if (note.taken()) s_note = 1;
   }
-  if (!alive && !s_refused) atomicExch(p.status, PAT_ERR_TIMEOUT);
-  __syncwarp();
   // every warp comes here, also after a failed wait: tensor memory is given back, and no CTA of a pair leaves while the other
   // may still signal its barriers.  A CTA that has received all partial sums is sent nothing more.
   if (!met) cluster_wait();
   if (CG == 2 && !left) cluster_arrive();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (!alive && !s_refused) atomicExch(p.status, PAT_ERR_TIMEOUT);
   auto give_time = [] {                                // 20 us: more than a copy or a store in flight takes
     const unsigned long long t0 = global_ns();
     while (global_ns() - t0 < 20000ull) {}
   };
-  const bool failed = s_abort != 0;
+  const bool failed = s_abort != 0 && !(ROWS8 && s_plain);  // (without the dense form nothing has been copied that could still arrive)
   if (failed) give_time();                             // copies that the other CTA of a pair did not arm
   if (CG == 2) {
     cluster_wait();
-  } else if (failed && clustered) {
+  } else if (s_abort != 0 && clustered) {
     cluster_arrive();
     cluster_wait();
   }
   if (failed && p.parts > 1) give_time();              // what the others had sent by then
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == W_MMA) free_columns<CG>(tmem);
-  if ((s_note && !failed) || (ROWS8 && s_plain)) {
+  if ((s_note && s_abort == 0) || (ROWS8 && s_plain)) {
     const bool whole = CG == 2 || p.parts == 1;
     renew_results<false, CG>(p, unit, n_units, CG == 2 ? (int)rank : 0, whole ? 0 : first_column<false>(p, (int)rank),
                              whole ? p.BN : first_column<false>(p, (int)rank + 1), ROWS8 && s_plain != 0);

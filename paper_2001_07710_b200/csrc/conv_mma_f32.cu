@@ -40,7 +40,7 @@ constexpr int UNITS = A_ROWS * 4 / (LOAD_WARPS * 32);      // (position, 8 chann
 static_assert(TILE + 2 * MAX_P + 2 <= A_ROWS, "a tile's rows fit a stage");
 constexpr int ST_BYTES = 256 * 128;
 constexpr int OFF_RING = 1024, RING_BYTES = 198656, OFF_ST = OFF_RING + RING_BYTES, SMEM_BYTES = OFF_ST + ST_BYTES;
-static_assert(SMEM_BYTES <= 232448 && OFF_ST % 1024 == 0, "shared memory budget of one SM");
+static_assert(SMEM_BYTES <= 232448 && OFF_ST % 1024 == 0 && OFF_RING == RING_AT && SMEM_BYTES == RING_TO, "shared memory budget of one SM");
 static_assert(SMEM_BYTES - OFF_RING >= (128 + MAX_PARTS_MMA * kPer<true>) * TILE * 4, "the partial sums of 128 filters fit");
 constexpr int BUF_COLS = 256;              // tensor memory: two buffers of 128 columns of main and 128 of small products
 
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
               if (!FOURS || c + 4 < p.C) v[j][1] = src[1];
             }
           }
-          if (!mbar_wait<20>(empty_a(slot), par, abort_flag, p.wait_ns)) alive = false;
+          if ((FOURS && pl == 0 && cb == cb0 && no_dense_form(p)) || !mbar_wait<20>(empty_a(slot), par, abort_flag, p.wait_ns)) alive = false;
           if (!__all_sync(0xFFFFFFFFu, alive)) { alive = false; break; }
           const uint32_t st = sbase + OFF_RING + (uint32_t)slot * p.a_bytes;
 #pragma unroll
@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
   } else if (warp == W_MMA) {
     // =========================================================================== multiply-adds (even CTA of a pair)
     // warp-uniform values and control flow, one elected lane issues (see conv_mma_f16.cu)
+    if (FOURS) alive = __all_sync(0xFFFFFFFFu, !no_dense_form(p)) != 0;
     if (leader) {
       const bool el = elect_one();
       int sa = 0, sb = 0, buf = 0;
@@ -353,10 +354,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
     Note note;
     const float floor_at = p.act != 0 ? 0.0f : -INFINITY;       // the rectifier
-    const int n_chunks = cb1 - cb0;
+    const int n_chunks = FOURS && no_dense_form(p) ? 0 : cb1 - cb0;
     int buf = 0;
     uint32_t pf = 0u;
     for (int item = unit; item < p.items && alive; item += n_units) {
+      if (FOURS && n_chunks == 0) break;
       const int tg = p.d_groups.div(item), g = item - tg * p.groups;
       const int m0 = (CG * tg + (int)side) * p.mstep;
       float acc[4][16];
@@ -432,32 +434,32 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_conv_mma_f32(const __grid_const
     }
     if (note.taken()) s_note = 1;
   }
-  if (!alive && !s_refused) atomicExch(p.status, PAT_ERR_TIMEOUT);
-  __syncwarp();
   // every warp comes here, also after a failed wait: tensor memory is given back, and no CTA of a pair leaves while the other
   // may still signal its barriers.  A CTA that has received all partial sums is sent nothing more.
   if (!met) cluster_wait();
   if (CG == 2 && !left) cluster_arrive();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (!alive && !s_refused) atomicExch(p.status, PAT_ERR_TIMEOUT);
   auto give_time = [] {                                // 20 us: more than a copy or a store in flight takes
     const unsigned long long t0 = global_ns();
     while (global_ns() - t0 < 20000ull) {}
   };
-  const bool failed = s_abort != 0;
+  const bool failed = s_abort != 0 && !(FOURS && s_plain);  // (without the dense form nothing has been copied that could still arrive)
   if (failed) give_time();                             // copies that the other CTA of a pair did not arm
   if (CG == 2) {
     cluster_wait();
-  } else if (failed && clustered) {
+  } else if (s_abort != 0 && clustered) {
     cluster_arrive();
     cluster_wait();
   }
   if (failed && p.parts > 1) give_time();              // what the others had sent by then
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == W_MMA) free_columns<CG>(tmem);
-  if ((s_note && !failed) || (FOURS && s_plain)) {
+  if ((s_note && s_abort == 0) || (FOURS && s_plain)) {
     const bool whole = p.parts == 1;
-    renew_results<true, CG>(p, unit, n_units, (int)side, whole ? 0 : first_column<true>(p, (int)part), whole ? p.BN : first_column<true>(p, (int)part + 1), FOURS && s_plain != 0);
+    renew_results<true, CG>(p, unit, n_units, (int)side, whole ? 0 : first_column<true>(p, (int)part),
+                             whole ? p.BN : first_column<true>(p, (int)part + 1), FOURS && s_plain != 0);
   }
 }
 

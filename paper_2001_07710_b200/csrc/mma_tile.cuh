@@ -13,8 +13,10 @@
 // taps that read it, again by constant shifts.
 #pragma once
 #include <algorithm>
+#include <type_traits>
 #include <cuda.h>
 #include "conv_tile.cuh"
+#include "plain_tile.cuh"
 
 namespace pat {
 namespace tmma {
@@ -31,6 +33,7 @@ constexpr int SUB = 128;                   // rows of one accumulator
 constexpr int MAX_P = 62;                  // positions per row
 constexpr int EPI_WARPS = 8;
 constexpr uint32_t TMEM_COLS = 512;
+constexpr int RING_AT = 1024, RING_TO = 232448;      // shared memory behind the barriers
 
 // What the kernels' parameter blocks have in common.
 struct Geometry {
@@ -255,7 +258,8 @@ __device__ __forceinline__ bool blob_matches_warp(const Geometry& p) {
   return __all_sync(0xFFFFFFFFu, ok) != 0;
 }
 
-// The blob holds no dense form, see dense_form_end: the results are formed from the packed kept taps alone.
+// The blob holds no dense form, see dense_form_end: the results are formed from the packed kept taps alone (plain_results).  Every
+// role finds that out for itself, while it waits for its first data: a wait that is given up takes 130 us to notice it.
 __device__ __forceinline__ bool no_dense_form(const Geometry& p) { return p.dense_end != 0 && p.hdr->total_bytes < p.dense_end; }
 
 // Output pixel of position m: index (n Ho + y) Wo + x, or -1 for padding positions.
@@ -348,10 +352,144 @@ __device__ __forceinline__ void store_one(const Geometry& p, size_t at, float v)
   if constexpr (F32) static_cast<float*>(p.y)[at] = v;
   else static_cast<__half*>(p.y)[at] = __float2half_rn(v);
 }
+// All results of a layer whose blob holds no dense form, by all threads of all blocks: the tiles of the generic kernel (see
+// conv_generic.cu: 8 x 32 outputs, four filters a warp, 16 channels staged at a time) by teams of warps, so that some stage while
+// others multiply.  The sums are those of that kernel, in its order.  Bound by staging and by reads of shared memory; a team has as
+// many warps as the layer has fours of filters, up to half of the block: what a stage brings then feeds most.  14 or 18 warps a block
+// instead of 24 a multiprocessor: 0.5 - 1.4 of the generic kernel's times (28x28x260 -> 256, batch 32, keep 1/4, fp16 725 us, 650
+// there, fp32 744, 654; 224x224x36 -> 64, batch 4, fp32 231, 167; 112x112x28 -> 8, batch 16, fp16 39, 73).  A lane per result that
+// gathers its own taps, as renew_results does it, took 36900 us for the first one.  Every role looks for the dense form itself, while it
+// waits for its first data: a wait that is given up takes 130 us to notice it.
+__device__ __forceinline__ void four_floats(const float4& a, float (&v)[4]) { v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; }
+__device__ __forceinline__ void four_floats(const uint2& a, float (&v)[4]) {
+  const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&a.x)), hi = __half22float2(*reinterpret_cast<const __half2*>(&a.y));
+  v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
+}
+constexpr int MAX_TEAMS = 9, TEAM_BARRIER = 3;           // first of the teams' named barriers
+template <bool F32, int STRIDE>
+__device__ __forceinline__ void plain_results(const Geometry& p, unsigned char* smem, int bytes) {
+  using T = typename std::conditional<F32, float, __half>::type;
+  using Four = typename std::conditional<F32, float4, uint2>::type;
+  using G = plain::Geo<STRIDE>;
+  using plain::TH; using plain::TW; using plain::RF; using plain::CB;
+  constexpr int STAGE = CB * G::PLANE;
+  const int warps = (int)blockDim.x >> 5, quads = (p.F + RF - 1) / RF;
+  int4* tapoff = reinterpret_cast<int4*>(smem);          // [K] offsets of the stored taps inside a plane
+  float* stages = reinterpret_cast<float*>(smem + 16 * 256);
+  const int room = min(MAX_TEAMS, (bytes - 16 * 256) / (STAGE * 4));
+  const int teams = min(room, max(2, warps / min(quads, warps / 2))), team = warps / teams, id = ((int)threadIdx.x >> 5) / team;
+  const BlobLayout L = blob_layout(p.F, p.C, p.K, p.n_keep, F32 ? PAT_F32 : PAT_F16);
+  const char* blob = reinterpret_cast<const char*>(p.hdr);
+  const int32_t* perm = reinterpret_cast<const int32_t*>(blob + L.xfilt);
+  const int32_t* tptr = reinterpret_cast<const int32_t*>(blob + L.tptr);
+  const uint32_t* tmeta = reinterpret_cast<const uint32_t*>(blob + L.tmeta);
+  const Four* tw4 = reinterpret_cast<const Four*>(blob + L.tw4);
+  const T* x = static_cast<const T*>(p.x);
+  for (int i = (int)threadIdx.x; i < p.K; i += (int)blockDim.x) {
+    unsigned m = p.masks[i];
+    int at[4];
+#pragma unroll
+    for (int tp = 0; tp < 4; ++tp, m &= m - 1u) {        // ascending bit order
+      const int b = __ffs(m) - 1;
+      at[tp] = (b / 3) * G::IWP + (b % 3);
+    }
+    tapoff[i] = make_int4(at[0], at[1], at[2], at[3]);
+  }
+  __syncthreads();
+  if (id >= teams) return;
+  const int lane = (int)threadIdx.x & 31, t = (int)threadIdx.x - id * team * 32, warp = t >> 5, threads = team * 32;
+  auto meet = [&] { asm volatile("barrier.sync %0, %1;" ::"r"(TEAM_BARRIER + id), "r"(threads) : "memory"); };
+  float* tile = stages + id * STAGE;
+  const int tiles_x = (p.Wo + TW - 1) / TW, tiles_y = (p.Ho + TH - 1) / TH, passes = (quads + team - 1) / team;
+  const long long n_units = (long long)p.N * tiles_y * tiles_x * passes;
+  for (long long unit = (long long)blockIdx.x * teams + id; unit < n_units; unit += (long long)gridDim.x * teams) {
+    const long long tl = unit / passes, ny = tl / tiles_x;
+    const int q0 = ((int)(unit - tl * passes) * team + warp) * RF;
+    const int n = (int)(ny / tiles_y), oy0 = (int)(ny - (long long)n * tiles_y) * TH, ox0 = (int)(tl - ny * tiles_x) * TW;
+    const int iy0 = oy0 * STRIDE - 1, ix0 = ox0 * STRIDE - 1;
+    float acc[RF][TH];
+#pragma unroll
+    for (int r = 0; r < RF; ++r)
+#pragma unroll
+      for (int k = 0; k < TH; ++k) acc[r][k] = 0.0f;
+    for (int cb = 0; cb < L.nct; ++cb) {
+      meet();                                            // the stage before has been read
+      for (int i = t; i < G::IH * G::IW; i += threads) {       // a position's 16 channels, in pieces of four (C is a multiple of that)
+        const int ty = i / G::IW, tx = i - ty * G::IW, yi = iy0 + ty, xi = ix0 + tx;
+        const bool in = yi >= 0 && yi < p.H && xi >= 0 && xi < p.W;
+        const T* src = x + (in ? (size_t)((n * p.H + yi) * p.W + xi) * p.C : 0) + cb * CB;
+        float* dst = tile + ty * G::IWP + tx;
+        constexpr int AT_ONCE = F32 ? 2 : 4;                   // loads of a thread in flight (more in fp32 takes registers from the kernel's own loops)
+#pragma unroll 1
+        for (int c0 = 0; c0 < CB / 4; c0 += AT_ONCE) {
+          Four piece[AT_ONCE];
+#pragma unroll
+          for (int u = 0; u < AT_ONCE; ++u) {
+            piece[u] = {};
+            if (in && cb * CB + 4 * (c0 + u) < p.C) piece[u] = *reinterpret_cast<const Four*>(src + 4 * (c0 + u));
+          }
+#pragma unroll
+          for (int u = 0; u < AT_ONCE; ++u) {
+            float v[4];
+            four_floats(piece[u], v);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) dst[(4 * (c0 + u) + k) * G::PLANE] = v[k];
+          }
+        }
+      }
+      meet();
+#pragma unroll
+      for (int r = 0; r < RF; ++r) {
+        const int q = q0 + r;
+        if (q >= p.F) continue;
+        const int kb = tptr[(size_t)q * (L.nct + 1) + cb], ke = tptr[(size_t)q * (L.nct + 1) + cb + 1];
+        // fp16: the next kernel's word and weights are read ahead
+        constexpr bool AHEAD = !F32;
+        uint32_t meta = 0u;
+        Four next = {};
+        if (AHEAD && kb < ke) { meta = tmeta[kb]; next = tw4[kb]; }
+        for (int k = kb; k < ke; ++k) {
+          if (!AHEAD) { meta = tmeta[k]; next = tw4[k]; }
+          const float* plane = tile + ((int)(meta & 0xFFFFu) - cb * CB) * G::PLANE + lane * STRIDE;
+          const int4 taps = tapoff[meta >> 16];
+          float w[4];
+          four_floats(next, w);
+          if (AHEAD && k + 1 < ke) { meta = tmeta[k + 1]; next = tw4[k + 1]; }
+          const int at[4] = {taps.x, taps.y, taps.z, taps.w};
+#pragma unroll
+          for (int tp = 0; tp < 4; ++tp) {
+            const float* src = plane + at[tp];
+#pragma unroll
+            for (int j = 0; j < TH; ++j) acc[r][j] = fmaf(w[tp], src[j * STRIDE * G::IWP], acc[r][j]);
+          }
+        }
+      }
+    }
+    const int ox = ox0 + lane;
+    if (ox < p.Wo) {
+#pragma unroll
+      for (int r = 0; r < RF; ++r) {
+        if (q0 + r >= p.F) continue;
+        const int f = perm[q0 + r];
+#pragma unroll
+        for (int k = 0; k < TH; ++k)
+          if (oy0 + k < p.Ho) store_one<F32>(p, (((size_t)n * p.Ho + oy0 + k) * p.Wo + ox) * p.F + f, p.act ? fmaxf(acc[r][k], 0.0f) : acc[r][k]);
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // The results that this block has stored - columns c_begin to c_end of its items - gone over by all its warps.  `all`: none has
-// been stored, every one is formed (layers without pooling only).
+// been stored, there is no dense form.
 template <bool F32, int CG>
 __device__ __noinline__ void renew_results(const Geometry& p, int unit, int n_units, int side, int c_begin, int c_end, bool all) {
+  if (all) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    if (p.stride == 1) plain_results<F32, 1>(p, smem + RING_AT, RING_TO - RING_AT);
+    else plain_results<F32, 2>(p, smem + RING_AT, RING_TO - RING_AT);
+    return;
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
   const int hw = p.Ws >> 1, n_out = p.act == 2 ? (p.d_P.div(p.mstep) >> 1) * hw : p.mstep;
   for (int item = unit; item < p.items; item += n_units) {
@@ -371,7 +509,7 @@ __device__ __noinline__ void renew_results(const Geometry& p, int unit, int n_un
         if (pixel < 0) continue;
         for (int f = f0 + lane; f < f1; f += 32) {
           const size_t at = (size_t)pixel * p.F + f;
-          const float old = all ? NAN : stored<F32>(p.y, at);
+          const float old = stored<F32>(p.y, at);
           if (old == old) continue;
           const float v = kept_taps<F32>(p, f, nn, yy, xx);
           store_one<F32>(p, at, p.act ? fmaxf(v, 0.0f) : v);       // (what pat_relu_maxpool makes of a NaN)
