@@ -263,9 +263,9 @@ __global__ void __launch_bounds__(threads_of(ROWS8), 1) k_conv_mma_f16(const __g
               }
             };
             if (!mbar_try_wait(empty_a(slot), par)) {
-              // the slot is still in use: bring the rows into L2 meanwhile
+              // the slot is still in use: bring the rows into L2 meanwhile (several from the row above the first image on: some are real)
               each([&](bool several, int x, int y, int n) {
-                if (y >= 0 && y < p.H && n < p.N) prefetch_4d(several ? &maps.rows : &maps.a, cb * KB, x, y, n);
+                if ((y >= 0 || several) && y < p.H && n < p.N) prefetch_4d(several ? &maps.rows : &maps.a, cb * KB, x, y, n);
               });
               if (!mbar_wait<20>(empty_a(slot), par, abort_flag, p.wait_ns)) { alive = false; break; }
             }
