@@ -106,7 +106,9 @@ int pat_project_static(const float *w, int F, int C, const uint16_t *masks, int 
 int64_t pat_project_static_max_kernels(void);
 
 /* Size in bytes of the packed blob of a layer (0 on invalid arguments).  A pure function of its
- * arguments, so no device-to-host transfer is ever needed to size a buffer. */
+ * arguments, so no device-to-host transfer is ever needed to size a buffer.  Layers with F a multiple of eight and C one of
+ * four hold their weights in dense form too (see pat_pack), 18 (fp16) or 54 (fp32) bytes per kernel of the layer, kept or not.
+ * Those with C an odd multiple of four once did not: with a buffer of the size from then pat_pack leaves the dense form out. */
 size_t pat_pack_size(int F, int C, int K, int64_t n_keep, int dtype);
 
 /* Compressed, re-ordered weight storage (Section 6.2: filters with similar kernels are grouped,
@@ -150,12 +152,15 @@ int pat_unpack(const void *blob, int F, int C, const uint16_t *masks, int K, int
  * even).
  * F a multiple of eight, C one of four: the tensor cores run the dense form of the masked weights, zeros included.  An infinity or NaN
  * reaches the outputs whose kept taps read it and no others all the same: results that the zeros would make NaN are formed
- * again from the kept taps, which takes its time when there are many.
+ * again from the kept taps, which takes its time when there are many.  A blob without the dense form (C an odd multiple of four,
+ * packed when such layers had none or into a buffer of that size; the header's length tells) has its kept taps multiplied as in
+ * the generic kernel and about as fast: pack again for the tensor cores.
  *   blob     dev, written by pat_pack with the same (F, C, masks, K, n_keep, dtype)
  *   masks    host, the library the blob was packed with
  *   x        dev, NHWC [N][H][W][C], 16-byte aligned
  *   y        dev out, NHWC [N][Ho][Wo][F], 16-byte aligned, must not overlap x
- * Any F and C in 1..65535 is accepted; the others run a generic kernel. */
+ * Any F and C in 1..65535 is accepted; the others run a generic kernel, as do large images of few channels and filters (C an odd
+ * multiple of four up to 20), where it is faster. */
 int pat_conv3x3(const void *blob, int F, int C, const uint16_t *masks, int K, int64_t n_keep,
                 int dtype, const void *x, void *y, int N, int H, int W, int stride, void *stream);
 

@@ -540,7 +540,9 @@ extern "C" int pat_pack(const float* w_masked, const uint8_t* pattern_id, int F,
   if (!w_masked || !pattern_id || !blob) return set_error(PAT_ERR_INVALID_ARG, "pat_pack: null pointer");
   if (int rc = common_checks("pat_pack", F, C, masks, K, n_keep, dtype)) return rc;
   if (!aligned(blob, 256)) return set_error(PAT_ERR_ALIGN, "pat_pack: blob must be 256-byte aligned");
-  const BlobLayout L = blob_layout(F, C, K, n_keep, dtype);
+  BlobLayout L = blob_layout(F, C, K, n_keep, dtype);
+  // a buffer sized when such layers had no dense form, which stands behind everything else: the blob goes without
+  if (dense_form_end(L, C) && blob_bytes < L.total && blob_bytes >= L.dense) { L.total = L.dense; L.dense = 0; }
   if (blob_bytes < L.total) return set_error(PAT_ERR_WORKSPACE, "pat_pack: blob has %zu bytes, needs %zu", blob_bytes, L.total);
   int* status = status_word();
   if (!status) return set_error(PAT_ERR_CUDA, "pat_pack: cannot resolve the status word");

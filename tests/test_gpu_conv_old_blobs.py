@@ -61,6 +61,29 @@ def test_results(case, dtype):
 
 
 @pytest.mark.parametrize("dtype", ["f16", "f32"])
+@pytest.mark.parametrize("C,F", [(36, 40), (4, 8)])
+def test_a_buffer_of_the_former_size_is_packed_without_the_dense_form(C, F, dtype):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(C)
+    masks, n_keep = pc.pat_library_builtin(8), F * C // 2
+    pid, wm = pc.pat_project(torch.randn((F, C, 3, 3), generator=gen, device="cuda"), masks, n_keep)
+    full = pc.pat_pack(wm, pid, masks, n_keep, dtype)
+    size = full.numel() - (9 * 2 * (1 if dtype == "f16" else 3) * F * ((C + 7) // 8 * 8) + 255) // 256 * 256
+    buf = torch.full((size + 512,), 7, dtype=torch.uint8, device="cuda")
+    small = pc.pat_pack(wm, pid, masks, n_keep, dtype, blob=buf[:size])
+    assert bool((buf[size:] == 7).all()) and int(small[32:40].view(torch.int64)) == size
+    assert torch.equal(pc.pat_unpack(small, F, C, masks, n_keep, dtype), pc.pat_unpack(full, F, C, masks, n_keep, dtype))
+    x = torch.randn((2, 9, 10, C), generator=gen, device="cuda").to(torch.float16 if dtype == "f16" else torch.float32)
+    y, old = (pc.pat_conv3x3(b, F, C, masks, n_keep, dtype, x, 1) for b in (full, small))
+    assert pc.pat_query_status() == 0
+    # two sums of up to 2 C terms, rounded to fp16 each
+    mag = torch.nn.functional.conv2d(x.abs().permute(0, 3, 1, 2).double(), wm.abs().double(), padding=1).permute(0, 2, 3, 1)
+    assert bool(((y.double() - old.double()).abs() <= 4 * C * STEP * mag + (2 * F16_ROUND * y.double().abs() + 2.0 ** -24 if dtype == "f16" else 0.0)).all())
+    with pytest.raises(pc.PatError):
+        pc.pat_pack(wm, pid, masks, n_keep, dtype, blob=buf[:size - 256])
+
+
+@pytest.mark.parametrize("dtype", ["f16", "f32"])
 @pytest.mark.parametrize("N,H,C,F,stride", [(1, 56, 68, 64, 1), (8, 28, 260, 256, 1), (2, 80, 20, 24, 2)])
 def test_time_is_that_of_the_generic_kernel(N, H, C, F, stride, dtype):
     """Two channels more take that kernel.  Measured 0.5 - 1.4 of its time; 10 - 57 times it when every result gathered its own taps."""
