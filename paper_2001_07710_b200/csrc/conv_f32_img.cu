@@ -222,6 +222,11 @@ __device__ __forceinline__ void one_kernel4f(float (&acc)[TR4][TC], uint32_t pla
 // Ring protocol: per work item nst stages of 8 channels, then two output stages whose slots
 // the consumers use as staging for the results - here twice (tile rows 0-1, then 2-3), with a block-wide barrier
 // after writing and after copying out the first pair of rows.
+// A consumer warp's wait, with one answer for all its lanes: they meet again at warp-wide instructions, tensor memory's among them, and
+// one that had given up by itself would leave the others waiting there.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait<0>(bar, parity, abort_flag)) != 0;
+}
 template <bool SPARSE, int NCODES, bool GENERIC>
 __device__ __forceinline__ void conv_body(const Params& p, unsigned char* smem) {
   constexpr int NS = SPARSE ? 3 : 2;
@@ -343,7 +348,7 @@ __device__ __forceinline__ void conv_body(const Params& p, unsigned char* smem) 
         for (int x = 0; x < TC; ++x) acc[y][x] = 0.0f;
       int c0, c1;
       const bool piece = piece_of(it_idx, c0, c1);
-      if (!mbar_wait<0>(slot_full(pslot), fpar, abort_flag)) { alive = false; break; }
+      if (!warp_wait(slot_full(pslot), fpar, abort_flag)) { alive = false; break; }
       uint32_t sl = slot0 + (uint32_t)pslot * SLOT;
       uint32_t pl0 = sl + offA;
       const uint32_t hw = lds32(sl + IMG_BYTES + (uint32_t)warp * 4u);
@@ -378,7 +383,7 @@ __device__ __forceinline__ void conv_body(const Params& p, unsigned char* smem) 
           if (lane == 0) mbar_arrive(slot_empty(pslot));
           if (++pslot == NS) { pslot = 0; fpar ^= 1u; }
           if (++cb == c1) break;
-          if (!mbar_wait<0>(slot_full(pslot), fpar, abort_flag)) { alive = false; break; }
+          if (!warp_wait(slot_full(pslot), fpar, abort_flag)) { alive = false; break; }
           sl = slot0 + (uint32_t)pslot * SLOT;
           pl0 = sl + offA;
           e = sl + IMG_BYTES + kBlockHeaderBytes + (cm >> kOpNextShift) * 16u;
@@ -413,8 +418,8 @@ __device__ __forceinline__ void conv_body(const Params& p, unsigned char* smem) 
       const uint32_t cposB = ((uint32_t)__ldg(p.xfilt + g_out * FG + FG - 1 - warp) & (uint32_t)(FG - 1)) * 4u;
       const int s0 = pslot, s1 = (pslot + 1 == NS) ? 0 : pslot + 1;
       const uint32_t par1 = (pslot + 1 == NS) ? (fpar ^ 1u) : fpar;
-      if (!mbar_wait<0>(slot_full(s0), fpar, abort_flag)) { alive = false; break; }
-      if (!mbar_wait<0>(slot_full(s1), par1, abort_flag)) { alive = false; break; }
+      if (!warp_wait(slot_full(s0), fpar, abort_flag)) { alive = false; break; }
+      if (!warp_wait(slot_full(s1), par1, abort_flag)) { alive = false; break; }
       const uint32_t ob0 = slot0 + (uint32_t)s0 * SLOT, ob1 = slot0 + (uint32_t)s1 * SLOT;
       const int txe_shift = (p.TXe == 4) ? 2 : (p.TXe == 2 ? 1 : 0);
       // tiles 16-31 sit one word further on: lanes l and l + 16 would otherwise store to the same banks
@@ -455,7 +460,7 @@ __device__ __forceinline__ void conv_body(const Params& p, unsigned char* smem) 
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(out_ready(0));
-        if (!mbar_wait<0>(out_ready(0), (uint32_t)round, abort_flag)) { alive = false; break; }
+        if (!warp_wait(out_ready(0), (uint32_t)round, abort_flag)) { alive = false; break; }
         // 14 pixels x 8 chunks of 4 channels per tile row: eight consecutive lanes write one pixel's 128 bytes
         const uint32_t slc = (uint32_t)(lane >> 3) * OUT_PITCH + (uint32_t)(lane & 7) * 16u;
 #pragma unroll 1
@@ -509,7 +514,7 @@ __device__ __forceinline__ void conv_body(const Params& p, unsigned char* smem) 
           // the second pair of rows overwrites the staging: every warp must have copied the first pair out
           __syncwarp();
           if (lane == 0) mbar_arrive(out_ready(1));
-          if (!mbar_wait<0>(out_ready(1), (uint32_t)(it_idx & 1), abort_flag)) { alive = false; break; }
+          if (!warp_wait(out_ready(1), (uint32_t)(it_idx & 1), abort_flag)) { alive = false; break; }
         }
       }
       if (!alive) break;
