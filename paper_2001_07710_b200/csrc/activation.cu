@@ -27,11 +27,11 @@ __device__ __forceinline__ uint4 relu_max(uint4 a, uint4 b, bool f16) {
   return r;
 }
 
-// chunks: 16-byte chunks per pixel (C * element size / 16).  One thread per (output pixel, chunk), chunks fastest, from the last one
-// down: what the kernel before this one wrote last is still in L2 when the tensor is larger than that, and so is what the next one
-// reads first.  Bound by the bytes when large, by the launch when small: a dependent launch, and divisions by multiplication
-// (Index = unsigned; long long beyond 2^31 chunks).  Convolution and pooling together: 12x20x32 -> 448, one image 8.5 -> 7.0 us,
-// 188x188x32 -> 96, batch 5 23.9 -> 21.1, 32x32x128, batch 128 33.6 -> 32.2.
+// chunks: 16-byte chunks per pixel (C * element size / 16).  One thread per (output pixel, chunk), chunks fastest.  Bound by the bytes
+// when large, by the launch when small: a dependent launch, and divisions by multiplication (Index = unsigned; long long beyond
+// 2^31 chunks, 34 GB of results: no test goes there).  Convolution and pooling together: 12x20x32 -> 448, one image 8.5 -> 7.0 us,
+// 188x188x32 -> 96, batch 5 23.9 -> 21.2, 32x32x128, batch 128 33.6 -> 31.9.  (From the last chunk to the first, for what is still in
+// L2: no difference at six shapes, 5 to 400 MB.)
 struct PoolSizes {
   int Wo, W, chunks;
   FastDiv d_Wo, d_chunks;
@@ -40,8 +40,7 @@ template <bool POOL, typename Index>
 __global__ void __launch_bounds__(256) k_relu_maxpool(const uint4* x, uint4* y, long long n_out, PoolSizes p, bool f16) {
   pdl_wait();
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += stride) {
-    const long long t = n_out - 1 - i;
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_out; t += stride) {
     if (!POOL) {
       const uint4 v = __ldcs(x + t);
       __stcs(y + t, relu_max(v, v, f16));
