@@ -11,8 +11,8 @@
 // memory: 44 clocks for 32 of arithmetic; its bytes take 126).
 //
 // The positions and shifts that make nine matrix products of a convolution are described in mma_tile.cuh.  A tile of 256
-// consecutive positions loads its input rows once and serves all nine taps from them (one TMA row copy per image row,
-// out-of-bounds rows and columns arrive as zeros); nine separate tap loads would need 64 B per clock and SM where
+// consecutive positions loads its input rows once and serves all nine taps from them (a TMA copy takes four rows of an image, one
+// where fewer are left; out-of-bounds rows and columns arrive as zeros); nine separate tap loads would need 64 B per clock and SM where
 // L2 delivers 36.  Stride 2: the tensor map's element strides pick the four planes.
 //
 // Work split.  CG = 2: a pair of CTAs (cta_group::2) shares a group of up to 256 filters: each CTA holds 256 positions (two
@@ -27,8 +27,9 @@
 //
 // Channels an odd multiple of four (ROWS8): activation rows start at multiples of 8 bytes only, which TMA does not take; four
 // warps then fill the same buffers with 8-byte cp.async (four: eight are no faster, the epilogue spills; 56x56x68 -> 200, batch 16:
-// 41 us, 72 channels through TMA 25: the copies' issue bounds it).  These layers ran the generic multiply-add kernel before:
-// 28x28x260 -> 256, batch 32 508 -> 47 us, 9x10x212 -> 152, batch 8 255 -> 13, 80x81x20 -> 24, stride 2, batch 2 64 -> 16.
+// 44 us, 72 channels through TMA 26: bound by the copies' issue and, in pairs, by an arrival across the cluster that every
+// loading warp makes a stage).  These layers ran the generic multiply-add kernel before (keep 1/4):
+// 28x28x260 -> 256, batch 32 650 -> 47 us, 9x10x212 -> 152, batch 8 118 -> 12, 80x81x20 -> 24, stride 2, batch 2 47 -> 14.
 //
 // Roles: warps 0-7 epilogue (tensor memory -> fp32 -> rectifier -> fp16 -> whole sectors of the output; pooled through shared memory), warp 8
 // copies activations, warp 9 weights, warp 10 issues the multiply-adds (in the even CTA of a pair).  Every wait is

@@ -16,8 +16,8 @@
 // shared memory bounds it (the operands of a 256 x 64 product take 44 clocks to read, the product 32), with stride 2 the
 // splitting of the activations (four planes for nine taps).
 //
-// Any multiple of four channels: activations are read 16 bytes at a time (28x28x260 -> 256, batch 32 499 us with the generic
-// kernel, 113 here; 66x62x84 -> 256, batch 2, 83 -> 22).
+// Any multiple of four channels: activations are read 16 bytes at a time (28x28x260 -> 256, batch 32, keep 1/4 654 us with the generic
+// kernel, 113 here; 56x56x68 -> 200, batch 16 286 and 80).
 //
 // Positions, taps and shifts: mma_tile.cuh.  A tile is 128 positions.  CG = 2: a pair of CTAs shares a group of up to 128
 // filters (half of the weights in each); CG = 1: one CTA per tile and group.  `parts`: the input channels are cut among
@@ -25,7 +25,8 @@
 //
 // Roles: warps 0-7 add up and write the results (warps 4-7 the upper half of the columns); warps 8-15 read the NHWC
 // activations, split them and write the three parts to shared memory (rows of 32 channels = 64 bytes, in the 64-byte swizzle
-// that the tensor core expects), one stage ahead; warp 16 copies weights (TMA); warp 17 issues the multiply-adds.
+// that the tensor core expects), one stage ahead; warp 16 copies weights (TMA); warp 17 issues the multiply-adds (in
+// the odd CTA of a pair it reports that CTA's stages to the even one).
 #include "mma_tile.cuh"
 
 namespace pat {
