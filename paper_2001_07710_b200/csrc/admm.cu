@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kBinThreads) k_argmax_binarize(const float* z,
 // kernels per mask are counted, per block in shared memory first.  The counters are zeroed by a kernel of their own; this
 // one is its programmatic dependent and does everything but the last additions before it waits for it.
 // FULL: the library is all 126 masks, so the best one holds the four largest squares (the whole call at 262144
-// kernels: 67 -> 10.5 us; a loop over 56 masks takes 21.5, so smaller libraries do not need a search of their own).
+// kernels: 67 -> 11.8 us; a loop over 56 masks takes 18.8, so smaller libraries do not need a search of their own).
 constexpr int kAssignThreads = 256, kFullK = 126;
 __global__ void __launch_bounds__(256) k_zero_counts(unsigned long long* counts, int K) {
   pdl_wait();
