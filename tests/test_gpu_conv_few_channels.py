@@ -33,4 +33,4 @@ def test_four_channels_take_no_longer_than_six(N, H, F, stride):
         y = pc.pat_conv3x3(blob, F, C, masks, n_keep, "f32", x, stride)
         return graph_ms(lambda: pc.pat_conv3x3(blob, F, C, masks, n_keep, "f32", x, stride, y=y), calls=10)
     ms(4)
-    assert ms(4) <= 1.1 * ms(6)
+    assert ms(4) <= 1.2 * ms(6)          # 0.95 measured; a fifth for two runs of one kernel that differ
